@@ -696,7 +696,8 @@ __global__ void k_combine_rows(int64_t n, int k, int nin, Ptrs6 W, const double*
 }
 
 // ---------------------------------------------------------------------------
-// Local solves: one warp per (subdomain l, column i) computes
+// FP32 local solves of windows above the register tiers: one warp per
+// (subdomain l, column i) computes
 //   w = (K_l - lambda_i M_l)^{-1} R_l rho_i
 // by a banded Cholesky factorisation streamed through a (B x B) window held
 // in shared memory (B = lower bandwidth + 1), with the forward substitution
@@ -707,11 +708,10 @@ __global__ void k_combine_rows(int64_t n, int k, int nin, Ptrs6 W, const double*
 // row j + B of the shifted band matrix into the freed slot.  Rows past n_l
 // are identity rows.  A pivot <= 0 sets err (Eq. (3.1) violated).
 // ---------------------------------------------------------------------------
-template <typename TP>
 __global__ void k_local_band(int npairs, int k, const int64_t* __restrict__ sub_ptr,
-                             const int32_t* __restrict__ sub_dofs, int B, const TP* __restrict__ bandK,
-                             const TP* __restrict__ bandM, const double* __restrict__ lam,
-                             const double* __restrict__ rho, TP* __restrict__ Lbuf, TP* __restrict__ wpk,
+                             const int32_t* __restrict__ sub_dofs, int B, const float* __restrict__ bandK,
+                             const float* __restrict__ bandM, const double* __restrict__ lam,
+                             const double* __restrict__ rho, float* __restrict__ Lbuf, float* __restrict__ wpk,
                              int32_t* err, int64_t rec_base) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x & 31;
@@ -719,47 +719,47 @@ __global__ void k_local_band(int npairs, int k, const int64_t* __restrict__ sub_
   const int pair = blockIdx.x * (blockDim.x >> 5) + wib;
   if (pair >= npairs) return;
   const int BB = B * B;
-  TP* W = reinterpret_cast<TP*>(smraw) + (size_t)wib * (BB + 3 * B);
-  TP* rw = W + BB;   // right-hand side window
-  TP* lc = rw + B;   // current column of L by slot
-  TP* xs = lc + B;   // solution window (backward sweep)
+  float* W = reinterpret_cast<float*>(smraw) + (size_t)wib * (BB + 3 * B);
+  float* rw = W + BB;   // right-hand side window
+  float* lc = rw + B;   // current column of L by slot
+  float* xs = lc + B;   // solution window (backward sweep)
   const int l = pair / k, i = pair % k;
   const int64_t off = sub_ptr[l];
   const int nl = (int)(sub_ptr[l + 1] - off);
   const int32_t* dofs = sub_dofs + off;
   const int b = B - 1;
-  const TP lm = (TP)lam[i];
-  TP* Lp = Lbuf + ((size_t)(off - rec_base) * k + (size_t)i * nl) * B;
-  auto aval = [&](int p, int q) -> TP {  // shifted local matrix entry, q <= p <= q + b
-    if (p >= nl) return (p == q) ? TP(1) : TP(0);
+  const float lm = (float)lam[i];
+  float* Lp = Lbuf + ((size_t)(off - rec_base) * k + (size_t)i * nl) * B;
+  auto aval = [&](int p, int q) -> float {  // shifted local matrix entry, q <= p <= q + b
+    if (p >= nl) return (p == q) ? float(1) : float(0);
     const size_t e = (size_t)(off + p) * B + (q - p + b);
     return bandK[e] - lm * bandM[e];
   };
   // initial window: rows 0..B-1
-  for (int e = lane; e < BB; e += 32) W[e] = TP(0);
+  for (int e = lane; e < BB; e += 32) W[e] = float(0);
   __syncwarp();
   for (int p = 0; p < B; ++p) {
     for (int e = lane; e <= b; e += 32) {
       int q = p - b + e;
       if (q < 0) continue;
-      TP v = aval(p, q);
+      float v = aval(p, q);
       W[(p % B) * B + (q % B)] = v;
       W[(q % B) * B + (p % B)] = v;
     }
     __syncwarp();
   }
-  for (int p = lane; p < B; p += 32) rw[p] = (p < nl) ? (TP)rho[(int64_t)dofs[p] * k + i] : TP(0);
+  for (int p = lane; p < B; p += 32) rw[p] = (p < nl) ? (float)rho[(int64_t)dofs[p] * k + i] : float(0);
   __syncwarp();
   for (int j = 0; j < nl; ++j) {
     const int s = j % B;
-    const TP piv = W[s * B + s];
-    if (!(piv > TP(0))) {
+    const float piv = W[s * B + s];
+    if (!(piv > float(0))) {
       if (lane == 0) atomicOr(err, 1);
       return;
     }
-    const TP inv = TP(1) / sqrt(piv);
-    for (int u = lane; u < B; u += 32) lc[u] = (u == s) ? TP(0) : W[u * B + s] * inv;
-    const TP yj = rw[s] * inv;
+    const float inv = float(1) / sqrt(piv);
+    for (int u = lane; u < B; u += 32) lc[u] = (u == s) ? float(0) : W[u * B + s] * inv;
+    const float yj = rw[s] * inv;
     __syncwarp();
     // L column j: slot 0 = 1/L_jj, slot t = L(j + t, j)
     for (int t = lane; t < B; t += 32) Lp[(size_t)j * B + t] = (t == 0) ? inv : lc[(j + t) % B];
@@ -786,31 +786,251 @@ __global__ void k_local_band(int npairs, int k, const int64_t* __restrict__ sub_
     const int pn = j + B;
     for (int e = lane; e <= b; e += 32) {
       int q = pn - b + e;  // q in j+1 .. j+B
-      TP v = aval(pn, q);
+      float v = aval(pn, q);
       W[s * B + (q % B)] = v;
       W[(q % B) * B + s] = v;
     }
-    if (lane == 0) rw[s] = (pn < nl) ? (TP)rho[(int64_t)dofs[pn] * k + i] : TP(0);
+    if (lane == 0) rw[s] = (pn < nl) ? (float)rho[(int64_t)dofs[pn] * k + i] : float(0);
     __syncwarp();
   }
   // backward substitution with L^T
-  for (int u = lane; u < B; u += 32) xs[u] = TP(0);
+  for (int u = lane; u < B; u += 32) xs[u] = float(0);
   __syncwarp();
   for (int j = nl - 1; j >= 0; --j) {
-    const TP* row = Lp + (size_t)j * B;
-    TP part = 0;
+    const float* row = Lp + (size_t)j * B;
+    float part = 0;
     for (int t = 1 + lane; t < B; t += 32) {
       if (j + t < nl) part += row[t] * xs[(j + t) % B];
     }
     part = warp_sum(part);
     if (lane == 0) {
-      TP xj = (wpk[(off + j) * k + i] - part) * row[0];
+      float xj = (wpk[(off + j) * k + i] - part) * row[0];
       xs[j % B] = xj;
       wpk[(off + j) * k + i] = xj;
     }
     __syncwarp();
   }
 }
+
+// ---------------------------------------------------------------------------
+// FP64 local solves: one CTA per (subdomain l, column i), the arithmetic of
+// k_local_band (column j eliminated with 1/L_jj = rsqrt(pivot), forward
+// substitution fused in, records as written there).  The FP64 pipe of this GPU
+// takes a warp instruction every 64 cycles per SM quarter, whatever its active
+// lanes, so instructions on that pipe are the bound and everything else
+// (shared memory, barriers) is nearly free beside them:
+//   - the symmetric window is kept once (packed lower triangle by slot index,
+//     entry (u, v), u >= v, at u (u + 1) / 2 + v; the right-hand sides are its last row) and updated by all warps over
+//     the flat list of its entries, full lanes in every instruction;
+//   - the warp that updates the next pivot forms its reciprocal root while the
+//     other warps do the rest of the update;
+//   - band rows and right-hand sides enter from registers loaded a step and a
+//     window period ahead;
+//   - backward, L^T x = y right-looking: the thread of a slot keeps the pending
+//     y of its row and streams its own record (contiguous, eight loads ahead),
+//     so a row costs one multiply, one fused multiply-add and one barrier.
+// 64 subdomains of 32 x 32 cells, 12 columns, window 37 (GB300): one warp per pair
+// on a full square window 10.27 ms, this kernel 2.9 ms (FP64 pipe 60 % busy; the
+// rest is the chain of a step and six pairs on some SMs against five on others)
+// ---------------------------------------------------------------------------
+constexpr int kPivotChunks = 7;
+__global__ void __launch_bounds__(192) k_local_band_f64(int k, const int64_t* __restrict__ sub_ptr,
+                                                        const int32_t* __restrict__ sub_dofs, int B,
+                                                        const double* __restrict__ bandK,
+                                                        const double* __restrict__ bandM,
+                                                        const double* __restrict__ lam,
+                                                        const double* __restrict__ rho, double* Lbuf, double* wpk,
+                                                        int32_t* err, int64_t rec_base) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ double s_inv, s_x[2];
+  __shared__ int s_bad;
+  const int NT = blockDim.x, tid = threadIdx.x, NR = B * (B + 1) / 2, NE = NR + B;
+  double* W = reinterpret_cast<double*>(smraw);  // [NE]: window, then the right-hand sides (row B)
+  double* lc = W + NE;                           // [B + 1] column of L by slot (0 at the pivot's), then y_j
+  double* ent = lc + B + 1;                      // [B + 1] entering band row by slot, then its right-hand side
+  double* rent = ent + B + 1;                    // [B] right-hand sides of the rows entering in this period
+  unsigned short* tab = reinterpret_cast<unsigned short*>(rent + B);  // [NE] (u << 8) | v
+  // slot of this thread (B: the right-hand side; threads past it only take part in the
+  // window update); the slots sit in other warps from one block to the next, so that the
+  // quarters of an SM share the per-slot work of its blocks
+  int u = tid + 32 * (blockIdx.x & 3);
+  u -= (u >= NT) ? NT : 0;
+  const bool own = u < B;
+  const int l = blockIdx.x / k, i = blockIdx.x % k;
+  const int64_t off = sub_ptr[l];
+  const int nl = (int)(sub_ptr[l + 1] - off);
+  const int32_t* dofs = sub_dofs + off;
+  const double* gK = bandK + (size_t)off * B;  // band row p at gK + p B, diagonal at B - 1
+  const double* gM = bandM + (size_t)off * B;
+  const double lm = lam[i];
+  double* Lp = Lbuf + ((size_t)(off - rec_base) * k + (size_t)i * nl) * B;
+  double* wp = wpk + off * k + i;
+  auto rhs = [&](int p) -> double { return (p < nl) ? rho[(int64_t)dofs[p] * k + i] : 0.0; };
+  // initial window: rows 0..B-1 (identity rows past nl)
+  for (int a = tid >> 5; a < B; a += NT >> 5)
+    for (int b = tid & 31; b <= a; b += 32) {
+      const int e = a * (a + 1) / 2 + b;
+      const size_t g = (size_t)a * B + (b - a + B - 1);
+      tab[e] = (unsigned short)((a << 8) | b);
+      W[e] = (a < nl) ? gK[g] - lm * gM[g] : ((a == b) ? 1.0 : 0.0);
+    }
+  double rn = 0.0, ek = 0.0, em = 0.0;
+  int ps = u - 1 + ((u == 0) ? B : 0);  // band position of this slot in the entering row
+  if (own) {
+    tab[NR + u] = (unsigned short)((B << 8) | u);
+    W[NR + u] = rhs(u);
+    rent[u] = rhs(B + u);
+    rn = rhs(2 * B + u);
+    if (B < nl) {
+      ek = gK[(size_t)B * B + ps];
+      em = gM[(size_t)B * B + ps];
+    }
+  }
+  if (tid == 0) s_bad = 0;
+  __syncthreads();
+  if (tid == 0) {
+    const double piv = W[0];
+    if (!(piv > 0.0)) {
+      s_bad = 1;
+      atomicOr(err, 1);
+    }
+    s_inv = rsqrt(piv);
+  }
+  __syncthreads();
+  if (s_bad) return;
+  const int nw = NT >> 5, nch = (NE + 31) / 32;
+  const int npc = max(1, (nch + kPivotChunks) / nw - kPivotChunks);
+  int role = (tid >> 5) + (blockIdx.x >> 2) % nw;  // 0: the warp of the pivot
+  role -= (role >= nw) ? nw : 0;
+  for (int j = 0, s = 0; j < nl; ++j) {
+    // column j of L and y_j, the record, the entering row j + B
+    if (u <= B) {
+      const double inv = s_inv;
+      const int hi = max(u, s), lo = min(u, s);
+      const double c = W[hi * (hi + 1) / 2 + lo] * inv;
+      lc[u] = (u == s) ? 0.0 : c;
+      if (own) {
+        int t = u - s;
+        t += (t < 0) ? B : 0;
+        Lp[(size_t)j * B + t] = (u == s) ? inv : c;
+        ent[u] = (j + B < nl) ? ek - lm * em : ((u == s) ? 1.0 : 0.0);
+        ps = (ps == 0) ? B - 1 : ps - 1;
+        if (j + 1 + B < nl) {
+          ek = gK[(size_t)(j + 1 + B) * B + ps];
+          em = gM[(size_t)(j + 1 + B) * B + ps];
+        }
+      } else {
+        ent[B] = rent[s];
+        wp[(size_t)j * k] = c;
+      }
+    }
+    __syncthreads();
+    // rank-one update by chunks of 32 entries; the pivot's slot takes the entering row.  One
+    // warp (another one each step) updates the next pivot's chunk first and forms its
+    // reciprocal root, which costs as much of the pipe as kPivotChunks chunks, so it takes
+    // that many fewer of the others
+    const int sn = (s + 1 == B) ? 0 : s + 1;
+    const int ep = sn * (sn + 1) / 2 + sn;  // the next pivot
+    // chunks r0, r0 + dr, ... (below r1) after the pivot's: the operands of all first
+    auto update = [&](auto count, int r0, int dr, int r1) -> double {
+      constexpr int N = decltype(count)::value;
+      int e[N], src[N];
+      double ca[N], cb[N], w[N], en[N];
+#pragma unroll
+      for (int c = 0; c < N; ++c) {
+        const int r = r0 + c * dr;
+        int q = ep / 32 + r;
+        q -= (q >= nch) ? nch : 0;
+        e[c] = q * 32 + (tid & 31);
+        if (r >= r1 || e[c] >= NE) e[c] = -1;
+        const int uv = tab[max(e[c], 0)];
+        const int a = uv >> 8, b = uv & 255;
+        src[c] = (a == s) ? b : ((b == s) ? a : -1);
+        ca[c] = lc[a];
+        cb[c] = lc[b];
+        w[c] = W[max(e[c], 0)];
+        en[c] = ent[max(src[c], 0)];
+      }
+#pragma unroll
+      for (int c = 0; c < N; ++c) {
+        w[c] = fma(-ca[c], cb[c], w[c]);
+        w[c] = (src[c] >= 0) ? en[c] : w[c];
+        if (e[c] >= 0) W[e[c]] = w[c];
+      }
+      return w[0];
+    };
+    if (role == 0) {
+      const double pv = update(std::integral_constant<int, 1>(), 0, 1, 1);
+      if ((tid & 31) == ep % 32) {
+        if (!(pv > 0.0)) {
+          s_bad = 1;
+          atomicOr(err, 1);
+        }
+        s_inv = rsqrt(pv);
+      }
+      for (int r = 1; r < npc; r += 4) update(std::integral_constant<int, 4>(), r, 1, npc);
+    } else {
+      for (int r = npc + role - 1; r < nch; r += 4 * (nw - 1))
+        update(std::integral_constant<int, 4>(), r, nw - 1, nch);
+    }
+    role = (role == 0) ? nw - 1 : role - 1;
+    if (sn == 0 && own) {
+      rent[u] = rn;
+      rn = rhs(j + 1 + 2 * B + u);
+    }
+    __syncthreads();
+    if (s_bad) return;
+    s = sn;
+  }
+  // backward substitution: slot u holds row q (q mod B = u), the pending y of which takes
+  // -L(j, q) x_j from every later row j; record q is read from entry B - 1 down to 1/L_qq
+  constexpr int PF = 8;
+  int t = 0, q = -1;  // entry and row of this thread's next load
+  double y = 0.0, yn = 0.0, ring[PF];
+  auto next = [&]() -> double {
+    const double v = (q >= 0) ? Lp[(size_t)q * B + t] : 0.0;
+    if (--t < 0) {
+      t = B - 1;
+      q -= B;
+    }
+    return v;
+  };
+  int row = -1;  // row held by this slot
+  if (own) {
+    t = (nl - 1) % B - u;
+    t += (t < 0) ? B : 0;
+    q = row = nl - 1 - t;
+    y = (row >= 0) ? wp[(size_t)row * k] : 0.0;
+    yn = (row >= B) ? wp[(size_t)(row - B) * k] : 0.0;
+  }
+#pragma unroll
+  for (int r = 0; r < PF; ++r) ring[r] = next();
+  if (own && row == nl - 1) s_x[(nl - 1) & 1] = y * ring[0];
+  for (int jb = nl - 1; jb >= 0; jb -= PF) {
+#pragma unroll
+    for (int r = 0; r < PF; ++r) {
+      const int j = jb - r;
+      if (j < 0) break;
+      __syncthreads();
+      if (own) {
+        const double xj = s_x[j & 1];
+        if (row == j) {
+          wp[(size_t)j * k] = xj;
+          y = yn;
+          row -= B;
+          yn = (row >= B) ? wp[(size_t)(row - B) * k] : 0.0;
+          // window of one row: the entering row is the next pivot
+          if (B == 1 && j > 0) s_x[(j - 1) & 1] = y * ring[(r + 1) % PF];
+        } else {
+          y = fma(-ring[r], xj, y);
+          if (row == j - 1) s_x[(j - 1) & 1] = y * ring[(r + 1) % PF];
+        }
+      }
+      ring[r] = next();
+    }
+  }
+}
+
 
 
 // ---------------------------------------------------------------------------
@@ -3098,21 +3318,22 @@ int launch_local(Handle& h, const double* rho, const double* lam, int mode) {
 #undef BPJD_LOCAL_TILE
 #undef BPJD_LOCAL_WIDE
       } else {
-        const size_t esz = f32 ? sizeof(float) : sizeof(double);
-        const size_t per_warp = (size_t)(B * B + 3 * B) * esz;
-        int wpb = (int)std::max<size_t>(1, std::min<size_t>(4, (200 * 1024) / per_warp));
-        size_t sm = per_warp * wpb;
-        int blocks = (npairs_c + wpb - 1) / wpb;
         if (f32) {
-          allow_dynamic_smem((const void*)k_local_band<float>);
-          k_local_band<float><<<blocks, 32 * wpb, sm, h.stream>>>(npairs_c, k, sptr, h.sub_dofs, B, h.bandKf,
-                                                                  h.bandMf, lam, rho, (float*)h.Lbuf,
-                                                                  (float*)h.wpk, h.derr, rec_base);
+          const size_t per_warp = (size_t)(B * B + 3 * B) * sizeof(float);
+          int wpb = (int)std::max<size_t>(1, std::min<size_t>(4, (200 * 1024) / per_warp));
+          size_t sm = per_warp * wpb;
+          int blocks = (npairs_c + wpb - 1) / wpb;
+          allow_dynamic_smem((const void*)k_local_band);
+          k_local_band<<<blocks, 32 * wpb, sm, h.stream>>>(npairs_c, k, sptr, h.sub_dofs, B, h.bandKf, h.bandMf, lam,
+                                                           rho, (float*)h.Lbuf, (float*)h.wpk, h.derr, rec_base);
         } else {
-          allow_dynamic_smem((const void*)k_local_band<double>);
-          k_local_band<double><<<blocks, 32 * wpb, sm, h.stream>>>(npairs_c, k, sptr, h.sub_dofs, B, h.bandK,
-                                                                   h.bandM, lam, rho, (double*)h.Lbuf,
-                                                                   (double*)h.wpk, h.derr, rec_base);
+          // four warps (one per SM quarter), six when the window has more rows
+          const int nt = std::max(128, (B + 32) / 32 * 32);
+          const size_t ne = (size_t)B * (B + 1) / 2 + B;
+          const size_t sm = (ne + 3 * B + 2) * sizeof(double) + ne * sizeof(unsigned short);
+          allow_dynamic_smem((const void*)k_local_band_f64);
+          k_local_band_f64<<<npairs_c, nt, sm, h.stream>>>(k, sptr, h.sub_dofs, B, h.bandK, h.bandM, lam, rho,
+                                                           (double*)h.Lbuf, (double*)h.wpk, h.derr, rec_base);
         }
       }
     }
@@ -3142,8 +3363,8 @@ int prime_kernel_attributes(Handle& h) {
     case 152: tier(std::integral_constant<int, 152>()); break;
     default: break;
   }
-  allow_dynamic_smem((const void*)k_local_band<float>);
-  allow_dynamic_smem((const void*)k_local_band<double>);
+  allow_dynamic_smem((const void*)k_local_band);
+  allow_dynamic_smem((const void*)k_local_band_f64);
   return (int)cudaGetLastError();
 }
 

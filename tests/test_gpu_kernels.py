@@ -1,0 +1,78 @@
+"""Kernels at the sizes where their tiles, windows and dispatch rules end, through the C ABI."""
+
+import numpy as np
+import pytest
+import scipy.linalg as la
+import scipy.sparse as sp
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+B = pytest.importorskip("paper_2203_06327_gb300.binding")
+
+DEV = "cuda"
+
+
+def _scipy(a):
+    return sp.csr_matrix((a.val, a.col_idx, a.row_ptr), shape=(a.n_rows, a.n_cols))
+
+
+def _reference(pb, part, rho, lam):
+    """Eq. (3.3) with dense factorisations."""
+    K, M, P = _scipy(pb.K), _scipy(pb.M), _scipy(pb.P)
+    k = len(lam)
+    w, Phi = la.eigh((P.T @ K @ P).toarray(), (P.T @ M @ P).toarray())
+    y = (Phi.T @ (P.T @ rho)) / (w[:, None] - lam[None, :])
+    y[:k] = 0.0
+    Z = P @ (Phi @ y)
+    for l in range(part.n_sub):
+        d = part.sub_dofs[part.sub_ptr[l]:part.sub_ptr[l + 1]]
+        Kl, Ml = K[d][:, d].toarray(), M[d][:, d].toarray()
+        for i in range(k):
+            Z[d, i] += la.solve(Kl - lam[i] * Ml, rho[d, i], assume_a="pos")
+    return Z
+
+
+def _parts(name):
+    """(problem, partition) with a given local window."""
+    if name == "window1":  # every third dof of a row of the grid: diagonal local matrices
+        pb = B.problem_create("p1_2d", (24, 18), (1.0, 0.751), (4, 3), 1)
+        n = pb.K.n_rows
+        lists = [np.arange(o, n, 3, dtype=np.int32) for o in range(3)]
+        lists = [d[(d // 23) % 2 == p] for d in lists for p in (0, 1)]
+    elif name == "short":  # subdomains of fewer dofs than the widest one's window
+        pb = B.problem_create("p1_2d", (24, 18), (1.0, 0.751), (4, 3), 1)
+        n = pb.K.n_rows
+        lists = [np.arange(0, 23 * 6, dtype=np.int32), np.arange(23 * 6, 23 * 6 + 5, dtype=np.int32),
+                 np.arange(n - 1, n, dtype=np.int32), np.arange(23 * 6, n, dtype=np.int32)]
+    else:  # strips as wide as the domain: window nx + 1
+        nx = int(name[6:]) - 1
+        pb = B.problem_create("p1_2d", (nx, 12), (1.0, 12.0 / nx), (nx, 12), 1)
+        n = pb.K.n_rows
+        # any full-rank interpolation serves: hats along x times hats along y on the dofs' own grid
+        ix, iy = np.arange(n) % (nx - 1) + 1, np.arange(n) // (nx - 1) + 1
+        hat = lambda t, c: np.maximum(0.0, 1.0 - np.abs(t - c) * 4)  # noqa: E731
+        cols = [hat(ix / nx, a / 4) * hat(iy / 12, b / 4) for b in (1, 2, 3) for a in (1, 2, 3)]
+        pb.P = B.CsrArrays.from_scipy(sp.csr_matrix(np.array(cols).T))
+        lists = [np.arange(0, (nx - 1) * 7, dtype=np.int32), np.arange((nx - 1) * 4, n, dtype=np.int32)]
+    ptr = np.concatenate([[0], np.cumsum([len(d) for d in lists])]).astype(np.int64)
+    return pb, B.PartitionArrays(ptr, np.concatenate(lists).astype(np.int32), None, 0)
+
+
+# FP64 windows at the ends of the kernel's mappings: one row, warp edges (32, 33), the last with four
+# warps (127) and the first beyond (128), the widest that fits (168); subdomains shorter than the window.
+# Tolerance as for the other FP64 preconditioner checks: 1e-10 of the largest entry (condition below 1e4).
+@pytest.mark.parametrize("name", ["window1", "short", "window32", "window33", "window127", "window128", "window168"])
+@pytest.mark.parametrize("k", [1, 3])
+def test_fp64_local_windows(name, k):
+    pb, part = _parts(name)
+    rng = np.random.default_rng(k)
+    lam = np.linspace(1.0, 12.0, k)  # below the lowest eigenvalue (at least 2 pi^2) of the pencil and its blocks
+    rho = rng.standard_normal((pb.K.n_rows, k))
+    ref = _reference(pb, part, rho, lam)
+    sv = B.Solver(pb.K, pb.M, pb.P, None, part, k, precision=B.FP64)
+    if name.startswith("window"):
+        assert sv.layout()["band_window"] == int(name[6:])
+    Z = torch.empty((sv.n, k), dtype=torch.float64, device=DEV)
+    sv.apply_preconditioner(torch.tensor(rho, device=DEV), torch.tensor(lam, device=DEV), Z)
+    assert np.abs(Z.cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref).max()
+    sv.close()

@@ -502,9 +502,9 @@ extern "C" int bpjd_setup(const bpjd_csr* A, const bpjd_csr* M, const bpjd_csr* 
     // band rows of the local matrices: FP32 (padded to the kernel tier) for FP32
     // local solves, FP64 otherwise
     if (h->local_f32()) {
-      const size_t W = (size_t)std::max(h->B, h->Bpad);
-      CK(dalloc(*h, &h->bandKf, (size_t)sum_nl * W));
-      CK(dalloc(*h, &h->bandMf, (size_t)sum_nl * W));
+      const size_t nb = band_floats(sum_nl, nsub, h->B, h->Bpad);
+      CK(dalloc(*h, &h->bandKf, nb));
+      CK(dalloc(*h, &h->bandMf, nb));
       if (h->same_pattern) {
         CKI(launch_band_fill(*h, h->A, h->M.val, nullptr, nullptr, h->bandKf, h->bandMf));
       } else {

@@ -74,7 +74,7 @@ struct Handle {
   double* bandK = nullptr;     // FP64 local solves: sum_nl x B, row p holds K_l(p, p-B+1 .. p)
   double* bandM = nullptr;
   float* bandKf = nullptr;     // FP32 local solves: sum_nl x max(B, Bpad), the same rows
-  float* bandMf = nullptr;     //   left-padded with zeros
+  float* bandMf = nullptr;     //   left-padded with zeros, or panels (band_panels)
 
   // ---- scratch
   void* Lbuf = nullptr;        // band factors of one chunk of subdomains (FP32 or FP64)
@@ -234,9 +234,16 @@ constexpr int kTransposeMaxCols = 24576;
 int launch_csr_transpose(const CsrDev& a, int64_t* rpT, int32_t* ciT, double* valT, cudaStream_t s);
 int launch_band_width(Handle& h, const CsrDev& c, int32_t* bw);
 int launch_split_values(const double* v, int64_t nnz, float2* out, cudaStream_t s);
+// tiers whose FP32 bands are stored by column panels (k_band_panels) instead of by rows,
+// and the floats that the bands of one matrix take
+inline bool band_panels(int bpad) { return bpad == 64 || bpad == 96 || bpad == 152; }
+inline size_t band_floats(int64_t sum_nl, int nsub, int B, int bpad) {
+  if (band_panels(bpad)) return (size_t)(sum_nl + 7 * (int64_t)nsub) * (bpad + 8);
+  return (size_t)sum_nl * (B > bpad ? B : bpad);
+}
 // band rows of the local matrices of c (and of a second matrix with c's pattern,
-// values val2): FP32 rows of width max(B, Bpad) into outf / outf2 when outf is
-// set, else FP64 rows of width B into out / out2
+// values val2): FP32 rows of width max(B, Bpad), or panels, into outf / outf2 when outf
+// is set, else FP64 rows of width B into out / out2
 int launch_band_fill(Handle& h, const CsrDev& c, const double* val2, double* out, double* out2, float* outf,
                      float* outf2);
 int launch_galerkin(const CsrDev& A, const CsrDev& Msp, const CsrDev& P, const CsrDev& PT, double* KH,

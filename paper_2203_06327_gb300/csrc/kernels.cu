@@ -1436,36 +1436,50 @@ __global__ void __launch_bounds__(128, (BMAX <= 40) ? 3 : 2) k_local_factor_mma(
 }
 
 // ---------------------------------------------------------------------------
-// Local solves, forward phase, blocked, for wide windows (B_pad = 64 or 96,
-// e.g. 3-D subdomains): one CTA per (subdomain, shift) with one thread per
-// window row (W = B_pad + 8 rows, NW = W / 32 rounded up warps).  The window
-// lives (negated) in m16n8k8 accumulator tiles; warp w owns the column tiles
-// ct = w, w + NW, ... of every row tile.  Per block step of eight columns:
-//   1. the warp owning the pivot column block writes it to shared memory;
-//   2. every thread reads its row of the panel and the 8 x 8 diagonal block,
-//      factorises the diagonal block redundantly in registers and solves for
-//      its own row of L (no barrier per column), eliminating its right-hand
-//      side entry; pivot rows store 1/L_jj, all rows their L entries;
-//   3. the L panel returns to shared memory and each warp applies the
-//      trailing update W <- W - L L^T to its tiles (TF32 head/tail split);
-//   4. each warp writes the entering band rows into its column tiles (values
-//      read from the FP32 band in global memory at the start of the step).
+// Local solves, forward phase, blocked, for wide windows (tiers 64, 96, 152:
+// 3-D subdomains and the clamped plate): one CTA per (subdomain, shift), banded
+// Cholesky eight columns at a time, left-looking.  The block step of columns
+// j0..j0+7 (column block J = j0 / 8) couples NBW = BMAX / 8 + 1 row blocks of
+// eight rows (relative blocks d = 0 .. NBW - 1):
+//   1. warp w accumulates the panel of row blocks 2w, 2w + 1 in one m16n8k8
+//      tile: minus the shifted band entries (read a step ahead) plus
+//      L(R, b) L(J, b)^T over the earlier column blocks b in ascending order,
+//      each product as tail x head + head x tail + head x head in TF32 (the
+//      operation order of a right-looking update, entry by entry); all but the
+//      last block's product run in the shadow of the previous step's 2;
+//   2. the last warp factorises the 8 x 8 diagonal block and solves for y;
+//   3. a thread per row forms its row of L (l = p L_dd^{-T}), eliminates its
+//      right-hand side, writes its entries of the eight records and leaves the
+//      TF32 head and tail of its row in shared memory for the later steps.
+// The history of L is kept in cells of 8 x 8 (row block R, column block b):
+// offset e = R - b <= NBW - 1, and cell (R, b) has the slot R mod e among the e
+// slots of its offset: when row block R becomes the pivot block its cells are
+// dead, and the cell of offset e is taken by (R + e, R).  So the triangle that
+// is live takes NBW (NBW - 1) / 2 cells and nothing moves.
+// A right-looking update holds the whole window in accumulators (168 registers,
+// two CTAs of 5 warps per SM at tier 96, one of 10 at 152) and needs its block
+// loop unrolled over the window, 13 to 20 copies that overflow the instruction
+// cache; here a thread holds four accumulators, the loop is rolled, and three
+// CTAs of 7 warps (tier 96) or two of 10 (152) share an SM.
 // Records and y have the layout of k_local_factor_mma, so k_local_backward
-// completes the solve.
+// completes the solve.  Measured (GB300, right-looking -> this): 5120 pairs of
+// window 92 5.2 -> 2.5 ms, 512 pairs of window 145 9.9 -> 4.1 ms; a step is a
+// chain of about 3700 cycles alone on an SM (the diagonal block 1650, its rows
+// 650), half the issue slots busy with three CTAs.  Taking each panel's products
+// in two half chains a step apart was 10 % slower (window 92) and 3 % (145).
 // ---------------------------------------------------------------------------
 template <int BMAX>
 struct WideShape {
   static constexpr int W = BMAX + 8;
-  static constexpr int NBW = W / 8;
-  static constexpr int RT = (W + 15) / 16;
-  static constexpr int CT = NBW;
-  // warps per CTA: one window row per thread, and at most three column tiles per warp
-  // (two above 128 rows, where the CTA has a whole SM: 80 accumulator registers)
-  static constexpr int CTMAX = (W > 128) ? 2 : 3;
-  static constexpr int NW = ((W + 31) / 32 > (CT + CTMAX - 1) / CTMAX) ? (W + 31) / 32 : (CT + CTMAX - 1) / CTMAX;
-  static constexpr int CTW = (CT + NW - 1) / NW;  // column tiles per warp (at most)
-  static constexpr int PSTR = 12;
-  static constexpr int MINB = (W > 128) ? 1 : 2;  // resident CTAs per SM the registers are sized for
+  static constexpr int NBW = W / 8;                 // row blocks of a panel
+  static constexpr int NW = (NBW + 1) / 2;          // warps: two row blocks each
+  static constexpr int CELL = 128;                  // floats of a cell: heads, then tails
+  static constexpr int NCELL = NBW * (NBW - 1) / 2;
+  static constexpr int PSTR = 12;                   // row stride of the panel buffer (bank-conflict free)
+  static constexpr int MINB = (BMAX == 64) ? 4 : (BMAX == 96) ? 3 : 2;
+  static constexpr size_t smem_floats = (size_t)NCELL * CELL + (size_t)NW * 16 * PSTR;
+  static_assert(NW * 32 >= W, "a thread per row");
+  static_assert(NCELL * CELL < 65536, "cell offsets in 16 bits");
 };
 
 template <int BMAX>
@@ -1473,14 +1487,17 @@ __global__ void __launch_bounds__(WideShape<BMAX>::NW * 32, WideShape<BMAX>::MIN
     int npairs, int k, const int64_t* __restrict__ sub_ptr, const int32_t* __restrict__ sub_dofs,
     const float* __restrict__ bandK, const float* __restrict__ bandM, const double* __restrict__ lam,
     const double* __restrict__ rho, float* __restrict__ Lbuf, float* __restrict__ wpk, int32_t* err,
-    int64_t rec_base) {
+    int64_t rec_base, int l0) {
   using S = WideShape<BMAX>;
-  constexpr int W = S::W, NBW = S::NBW, RT = S::RT, CT = S::CT, NW = S::NW, CTW = S::CTW, PSTR = S::PSTR;
-  static_assert(BMAX % 8 == 0 && CTW * 4 * RT <= 128, "window too wide for the register tiles");
-  __shared__ __align__(16) float pbuf[RT * 16 * PSTR];  // panel, then L operand; rows >= W stay zero
-  __shared__ float srhs[8];
-  const int tid = threadIdx.x, lane_id = tid & 31, wid = tid >> 5;
-  const int lane_g = lane_id >> 2, lane_q = lane_id & 3;
+  constexpr int W = S::W, NBW = S::NBW, NW = S::NW, PSTR = S::PSTR, CELL = S::CELL;
+  constexpr unsigned FULL = 0xffffffffu;
+  extern __shared__ __align__(16) float wsm[];
+  float* cells = wsm;                                     // [NCELL][CELL]
+  float* pbuf = wsm + (size_t)S::NCELL * CELL;            // [NW 16][PSTR] negated panel by relative row
+  __shared__ __align__(16) float sD[8][8];                // factor of the diagonal block (lower triangle)
+  __shared__ __align__(16) float sdinv[8], sy[8], srhs[8];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int g = lane >> 2, q = lane & 3;
   const int pair = blockIdx.x;
   if (pair >= npairs) return;
   const int l = pair / k, i = pair % k;
@@ -1490,159 +1507,193 @@ __global__ void __launch_bounds__(WideShape<BMAX>::NW * 32, WideShape<BMAX>::MIN
   const float lm = (float)lam[i];
   float* Lrec = Lbuf + ((size_t)(off - rec_base) * k + (size_t)i * nl) * BMAX;
   float* yout = wpk + off * k + i;
-  const float* gK = bandK + (size_t)off * BMAX;  // band row p at gK + p * BMAX, diagonal at BMAX - 1
-  const float* gM = bandM + (size_t)off * BMAX;
-  for (int e = tid; e < RT * 16 * PSTR; e += blockDim.x) pbuf[e] = 0.f;
-  // shifted entry (p, q), q <= p (identity rows beyond nl)
-  auto a0 = [&](int p, int q) -> float {
-    if (p >= nl) return (p == q) ? 1.f : 0.f;
-    const int d = p - q;
-    if (d > BMAX - 1 || q < 0) return 0.f;
-    const int e = BMAX - 1 - d;
-    return gK[(size_t)p * BMAX + e] - lm * gM[(size_t)p * BMAX + e];
-  };
+  // panel layout of the bands (k_band_panels): entry (row j0 + dr, column j0 + c) of column
+  // block J at (J W + dr) 8 + c, zeros outside the band, identity rows past nl
+  const int64_t pb = (off + 7 * (int64_t)(l + l0)) * W + (16 * w + g) * 8 + 2 * q;
+  const float* gK = bandK + pb;
+  const float* gM = bandM + pb;
   auto rhs = [&](int p) -> float { return (p < nl) ? (float)rho[(int64_t)dofs[p] * k + i] : 0.f; };
-  // initial window rows 0..W-1 (negated, both triangles) in this warp's column tiles
-  float acc[RT][CTW][4];
+  // band entries of this lane's accumulators in panel J: rows 16 w + g and + 8 (the last
+  // warp of an odd NBW has no second row block), columns 2 q and 2 q + 1
+  const int dr0 = 16 * w + g;
+  const int nJ = (nl + 7) >> 3;
+  float2 ek[2], em[2];
+  auto load_band = [&](int J) {
 #pragma unroll
-  for (int rt = 0; rt < RT; ++rt)
-#pragma unroll
-    for (int jl = 0; jl < CTW; ++jl)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int ct = wid + NW * jl;
-        const int u = rt * 16 + lane_g + 8 * (e >> 1), v = ct * 8 + 2 * lane_q + (e & 1);
-        acc[rt][jl][e] = (ct < CT && u < W) ? -((u >= v) ? a0(u, v) : a0(v, u)) : 0.f;
-      }
-  float r = (tid < W) ? rhs(tid) : 0.f;  // right-hand side of this thread's window row
+    for (int h = 0; h < 2; ++h) {
+      const bool ok = J < nJ && 2 * w + h < NBW;
+      ek[h] = ok ? *reinterpret_cast<const float2*>(gK + (int64_t)J * (8 * W) + 64 * h) : make_float2(0.f, 0.f);
+      em[h] = ok ? *reinterpret_cast<const float2*>(gM + (int64_t)J * (8 * W) + 64 * h) : make_float2(0.f, 0.f);
+    }
+  };
+  float acc[4];
+  auto start_panel = [&]() {  // minus the shifted band
+    acc[0] = fmaf(lm, em[0].x, -ek[0].x);
+    acc[1] = fmaf(lm, em[0].y, -ek[0].y);
+    acc[2] = fmaf(lm, em[1].x, -ek[1].x);
+    acc[3] = fmaf(lm, em[1].y, -ek[1].y);
+  };
+  // cells that lane D - 1 serves for the panel under way (block Jp, distance D of the earlier
+  // column block): row blocks Jp + 2 w and Jp + 2 w + 1 at offsets e0 and e0 + 1, slot
+  // (Jp - D) mod offset, and the pivot block at offset D, slot Jp mod D; Jp mod offset is
+  // advanced with Jp
+  const int D = lane + 1, e0 = 2 * w + D, e1 = e0 + 1;
+  int m0 = 0, m1 = 0, mb = 0;
+  uint32_t oa = 0;
+  int ob = 0;
+  auto cell_of = [](int e, int m) { return (e * (e - 1) / 2 + m) * CELL; };
+  auto advance = [&]() {
+    m0 = (m0 + 1 == e0) ? 0 : m0 + 1;
+    m1 = (m1 + 1 == e1) ? 0 : m1 + 1;
+    mb = (mb + 1 == D) ? 0 : mb + 1;
+    int x0 = m0 - D, x1 = m1 - D;
+    x0 += (x0 < 0) ? e0 : 0;
+    x1 += (x1 < 0) ? e1 : 0;
+    oa = (uint32_t)cell_of(e0, x0) | ((uint32_t)cell_of(e1, x1) << 16);  // below 2^16 for the cells that exist
+    ob = cell_of(D, mb);
+  };
+  struct Frag {
+    float2 h0, l0, h1, l1, hb, lb;
+  };
+  const float* cl = cells + g * 8 + 2 * q;
+  auto load_frag = [&](int d) -> Frag {
+    Frag f;
+    const uint32_t o = __shfl_sync(FULL, oa, d - 1);
+    const float* c0 = cl + (o & 0xffffu);
+    const float* c1 = cl + (o >> 16);
+    const float* cb = cl + __shfl_sync(FULL, ob, d - 1);
+    f.h0 = *reinterpret_cast<const float2*>(c0);
+    f.l0 = *reinterpret_cast<const float2*>(c0 + 64);
+    f.h1 = f.l1 = make_float2(0.f, 0.f);
+    if (2 * w + 1 + d < NBW) {
+      f.h1 = *reinterpret_cast<const float2*>(c1);
+      f.l1 = *reinterpret_cast<const float2*>(c1 + 64);
+    }
+    f.hb = *reinterpret_cast<const float2*>(cb);
+    f.lb = *reinterpret_cast<const float2*>(cb + 64);
+    return f;
+  };
+  auto add_frag = [&](const Frag& f) {
+    const uint32_t ah[4] = {__float_as_uint(f.h0.x), __float_as_uint(f.h1.x), __float_as_uint(f.h0.y),
+                            __float_as_uint(f.h1.y)};
+    const uint32_t al[4] = {__float_as_uint(f.l0.x), __float_as_uint(f.l1.x), __float_as_uint(f.l0.y),
+                            __float_as_uint(f.l1.y)};
+    mma_tf32(acc, al, __float_as_uint(f.hb.x), __float_as_uint(f.hb.y));
+    mma_tf32(acc, ah, __float_as_uint(f.lb.x), __float_as_uint(f.lb.y));
+    mma_tf32(acc, ah, __float_as_uint(f.hb.x), __float_as_uint(f.hb.y));
+  };
+  load_band(0);
+  start_panel();
+  load_band(1);
+  float r = (tid < W) ? rhs(tid) : 0.f;  // right-hand side of this thread's slot (row mod W)
+  int slot0 = 0;                         // j0 mod W
+  int jm = 0;                            // j0 mod BMAX
   bool bad = false;
-  int jm = 0;  // j0 mod BMAX
-  __syncthreads();
-  for (int c = 0; c * W < nl; ++c) {
-#pragma unroll
-    for (int sb = 0; sb < NBW; ++sb) {
-      const int j0 = c * W + 8 * sb;
-      if (j0 >= nl) break;
-      int zero;
-      asm volatile("mov.u32 %0, 0;" : "=r"(zero));
-      const int g = lane_g + zero, q = lane_q + zero, t = tid + zero;
-      // entering band rows j0 + W + g (this lane's row of the entering block) for the
-      // row part of this warp's column tiles, read now and written in step 4
-      const int pnew = j0 + W + g;
-      const bool realg = pnew < nl;
-      float ek[CTW][2], em[CTW][2];
-#pragma unroll
-      for (int jl = 0; jl < CTW; ++jl)
-#pragma unroll
-        for (int e2 = 0; e2 < 2; ++e2) {
-          const int ct = wid + NW * jl;
-          float kv = 0.f, mv = 0.f;
-          int pr = pnew, ps = -1;
-          if (ct < CT) {
-            if (ct != sb) {
-              // column slot ct 8 + 2 q + e2 holds row j0 + dv, dv = ((ct - sb) mod NBW) 8 + 2 q + e2
-              ps = ((ct - sb + NBW) % NBW) * 8 + e2 - 9 + 2 * q - g;
-            } else {
-              const int du2 = 2 * q + e2;
-              pr = (g >= du2) ? pnew : j0 + W + du2;  // the later row of the pair
-              ps = BMAX - 1 - ((g >= du2) ? g - du2 : du2 - g);
-            }
-          }
-          if (ps >= 0 && pr < nl) {
-            kv = gK[(size_t)pr * BMAX + ps];
-            mv = gM[(size_t)pr * BMAX + ps];
-          }
-          ek[jl][e2] = kv;
-          em[jl][e2] = mv;
-        }
-      const int d8 = t - 8 * sb;  // position of this row in the pivot block (0..7 there)
-      const float rnew = (d8 >= 0 && d8 < 8) ? rhs(pnew - g + d8) : 0.f;
-      // 1. pivot column block -> pbuf[slot][0..7]; pivot right-hand sides -> srhs
-      if (wid == sb % NW) {
-#pragma unroll
-        for (int rt = 0; rt < RT; ++rt) {
-          *reinterpret_cast<float2*>(pbuf + (rt * 16 + g) * PSTR + 2 * q) =
-              make_float2(acc[rt][sb / NW][0], acc[rt][sb / NW][1]);
-          *reinterpret_cast<float2*>(pbuf + (rt * 16 + g + 8) * PSTR + 2 * q) =
-              make_float2(acc[rt][sb / NW][2], acc[rt][sb / NW][3]);
-        }
-      }
-      if (d8 >= 0 && d8 < 8) srhs[d8] = r;
-      __syncthreads();
-      // 2. own row of the panel and the diagonal block, both negated back
-      int dr = t - 8 * sb;
-      dr += (dr < 0) ? W : 0;
-      const bool row_ok = t < W;
-      float p[8];
-      {
-        const float4 x0 = *reinterpret_cast<const float4*>(pbuf + (row_ok ? t : 0) * PSTR);
-        const float4 x1 = *reinterpret_cast<const float4*>(pbuf + (row_ok ? t : 0) * PSTR + 4);
-        p[0] = -x0.x; p[1] = -x0.y; p[2] = -x0.z; p[3] = -x0.w;
-        p[4] = -x1.x; p[5] = -x1.y; p[6] = -x1.z; p[7] = -x1.w;
-      }
-      float D[8][8];  // lower triangle used
+  for (int j0 = 0, J = 0; j0 < nl; j0 += 8, ++J) {
+    // this thread's row relative to j0, and the right-hand side that enters its slot
+    int dr = tid - slot0;
+    dr += (dr < 0) ? W : 0;
+    const bool row_ok = tid < W;
+    float rnew = 0.f;
+    if (row_ok && dr < 8) {
+      srhs[dr] = r;
+      rnew = rhs(j0 + W + dr);
+    }
+    // 1. the last column block's products complete the panel
+    if (J > 0 && 2 * w + 1 < NBW) add_frag(load_frag(1));
+    *reinterpret_cast<float2*>(pbuf + dr0 * PSTR + 2 * q) = make_float2(acc[0], acc[1]);
+    *reinterpret_cast<float2*>(pbuf + (dr0 + 8) * PSTR + 2 * q) = make_float2(acc[2], acc[3]);
+    __syncthreads();
+    const int mj = mb;  // J mod (lane + 1)
+    advance();
+    // 2. Cholesky of the diagonal block and y = L_dd^{-1} rhs (every lane of the last warp)
+    if (w == NW - 1) {
+      float Dm[8][8], dinv[8], yv[8];
 #pragma unroll
       for (int a = 0; a < 8; ++a) {
-        const float4 x0 = *reinterpret_cast<const float4*>(pbuf + (8 * sb + a) * PSTR);
-        const float4 x1 = *reinterpret_cast<const float4*>(pbuf + (8 * sb + a) * PSTR + 4);
-        D[a][0] = -x0.x; D[a][1] = -x0.y; D[a][2] = -x0.z; D[a][3] = -x0.w;
-        D[a][4] = -x1.x; D[a][5] = -x1.y; D[a][6] = -x1.z; D[a][7] = -x1.w;
+        const float4 x0 = *reinterpret_cast<const float4*>(pbuf + a * PSTR);
+        const float4 x1 = *reinterpret_cast<const float4*>(pbuf + a * PSTR + 4);
+        Dm[a][0] = -x0.x; Dm[a][1] = -x0.y; Dm[a][2] = -x0.z; Dm[a][3] = -x0.w;
+        Dm[a][4] = -x1.x; Dm[a][5] = -x1.y; Dm[a][6] = -x1.z; Dm[a][7] = -x1.w;
+        yv[a] = srhs[a];
       }
-      float yv[8];
-#pragma unroll
-      for (int a = 0; a < 8; ++a) yv[a] = srhs[a];
-      __syncthreads();  // pbuf and srhs are rewritten below
-      // Cholesky of the diagonal block (every thread), inverse diagonal in dinv
-      float dinv[8];
 #pragma unroll
       for (int cc = 0; cc < 8; ++cc) {
-        float s = D[cc][cc];
+        float s = Dm[cc][cc];
 #pragma unroll
-        for (int b = 0; b < cc; ++b) s = fmaf(-D[cc][b], D[cc][b], s);
+        for (int b = 0; b < cc; ++b) s = fmaf(-Dm[cc][b], Dm[cc][b], s);
         bad |= !(s > 0.f);
         const float inv = rsqrtf(s);
         dinv[cc] = inv;
-        D[cc][cc] = s * inv;
+        Dm[cc][cc] = s * inv;
 #pragma unroll
         for (int a = cc + 1; a < 8; ++a) {
-          float v = D[a][cc];
+          float v = Dm[a][cc];
 #pragma unroll
-          for (int b = 0; b < cc; ++b) v = fmaf(-D[a][b], D[cc][b], v);
-          D[a][cc] = v * inv;
+          for (int b = 0; b < cc; ++b) v = fmaf(-Dm[a][b], Dm[cc][b], v);
+          Dm[a][cc] = v * inv;
         }
       }
-      // y = L_dd^{-1} rhs of the pivot rows
 #pragma unroll
       for (int a = 0; a < 8; ++a) {
         float v = yv[a];
 #pragma unroll
-        for (int b = 0; b < a; ++b) v = fmaf(-D[a][b], yv[b], v);
+        for (int b = 0; b < a; ++b) v = fmaf(-Dm[a][b], yv[b], v);
         yv[a] = v * dinv[a];
       }
-      // own row of L: l = p L_dd^{-T}; for a pivot row (dr < 8) this reproduces row dr
-      // of L_dd, whose entries past the diagonal are cleared
+      if (lane == 0) {
+#pragma unroll
+        for (int a = 0; a < 8; ++a) {
+          *reinterpret_cast<float4*>(&sD[a][0]) = make_float4(Dm[a][0], Dm[a][1], Dm[a][2], Dm[a][3]);
+          *reinterpret_cast<float4*>(&sD[a][4]) = make_float4(Dm[a][4], Dm[a][5], Dm[a][6], Dm[a][7]);
+          sdinv[a] = dinv[a];
+          sy[a] = yv[a];
+          if (j0 + a < nl) yout[(size_t)(j0 + a) * k] = yv[a];
+        }
+      }
+    }
+    // the next panel: its band entries and the products of the column blocks before this one
+    start_panel();
+    load_band(J + 2);
+    {
+      const int dtop = min(J + 1, NBW - 1 - 2 * w);
+      if (dtop >= 2) {
+        Frag f = load_frag(dtop);
+        for (int d = dtop - 1; d >= 2; --d) {
+          const Frag n = load_frag(d);
+          add_frag(f);
+          f = n;
+        }
+        add_frag(f);
+      }
+    }
+    __syncthreads();
+    const int md = __shfl_sync(FULL, mj, max((dr >> 3) - 1, 0));  // J mod the row's offset
+    // 3. own row of L: l = p L_dd^{-T}; for a pivot row (dr < 8) this reproduces row dr of
+    // L_dd up to its diagonal
+    if (row_ok) {
       float lr[8];
+      {
+        const float4 x0 = *reinterpret_cast<const float4*>(pbuf + dr * PSTR);
+        const float4 x1 = *reinterpret_cast<const float4*>(pbuf + dr * PSTR + 4);
+        lr[0] = -x0.x; lr[1] = -x0.y; lr[2] = -x0.z; lr[3] = -x0.w;
+        lr[4] = -x1.x; lr[5] = -x1.y; lr[6] = -x1.z; lr[7] = -x1.w;
+      }
+      float dinv[8];
+      *reinterpret_cast<float4*>(&dinv[0]) = *reinterpret_cast<const float4*>(&sdinv[0]);
+      *reinterpret_cast<float4*>(&dinv[4]) = *reinterpret_cast<const float4*>(&sdinv[4]);
 #pragma unroll
       for (int cc = 0; cc < 8; ++cc) {
-        float v = p[cc];
+        float v = lr[cc];
+        const float4 d0 = *reinterpret_cast<const float4*>(&sD[cc][0]);
+        const float4 d1 = *reinterpret_cast<const float4*>(&sD[cc][4]);
+        const float Dr[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
 #pragma unroll
-        for (int b = 0; b < cc; ++b) v = fmaf(-lr[b], D[cc][b], v);
+        for (int b = 0; b < cc; ++b) v = fmaf(-lr[b], Dr[b], v);
         lr[cc] = v * dinv[cc];
       }
-      if (dr < 8) {
-#pragma unroll
-        for (int cc = 0; cc < 8; ++cc)
-          if (cc > dr) lr[cc] = 0.f;
-      } else {
-#pragma unroll
-        for (int cc = 0; cc < 8; ++cc) r = fmaf(-lr[cc], yv[cc], r);
-      }
-      if (!row_ok) {
-#pragma unroll
-        for (int cc = 0; cc < 8; ++cc) lr[cc] = 0.f;
-      }
       // records: column j0 + cc holds L(row, j0 + cc) at row mod BMAX, 1/L_jj at the pivot
-      if (row_ok) {
+      {
         int pos = jm + dr;
         pos -= (pos >= BMAX) ? BMAX : 0;
         pos -= (pos >= BMAX) ? BMAX : 0;
@@ -1653,74 +1704,35 @@ __global__ void __launch_bounds__(WideShape<BMAX>::NW * 32, WideShape<BMAX>::MIN
           if (j0 + cc < nl && tt >= 0 && tt < BMAX) rec[(size_t)cc * BMAX] = (tt == 0) ? dinv[cc] : lr[cc];
         }
       }
-      if (t == 0) {
+      if (dr < 8) {
+        r = rnew;
+      } else {
+        float yv[8];
+        *reinterpret_cast<float4*>(&yv[0]) = *reinterpret_cast<const float4*>(&sy[0]);
+        *reinterpret_cast<float4*>(&yv[4]) = *reinterpret_cast<const float4*>(&sy[4]);
+        float hi[8], lo[8];
 #pragma unroll
-        for (int cc = 0; cc < 8; ++cc)
-          if (j0 + cc < nl) yout[(size_t)(j0 + cc) * k] = yv[cc];
-      }
-      // 3. L panel -> pbuf, trailing update of this warp's tiles
-      if (row_ok) {
-        *reinterpret_cast<float4*>(pbuf + t * PSTR) = make_float4(lr[0], lr[1], lr[2], lr[3]);
-        *reinterpret_cast<float4*>(pbuf + t * PSTR + 4) = make_float4(lr[4], lr[5], lr[6], lr[7]);
-      }
-      __syncthreads();
-      uint32_t bh[CTW][2], bl[CTW][2];
-#pragma unroll
-      for (int jl = 0; jl < CTW; ++jl) {
-        const int ct = wid + NW * jl;
-        const int row = (ct < CT ? ct : 0) * 8 + g;
-        const float x0 = pbuf[row * PSTR + q], x1 = pbuf[row * PSTR + q + 4];
-        bh[jl][0] = to_tf32(x0);
-        bl[jl][0] = to_tf32(x0 - __uint_as_float(bh[jl][0]));
-        bh[jl][1] = to_tf32(x1);
-        bl[jl][1] = to_tf32(x1 - __uint_as_float(bh[jl][1]));
-      }
-#pragma unroll
-      for (int rt = 0; rt < RT; ++rt) {
-        float x[4];
-        x[0] = pbuf[(rt * 16 + g) * PSTR + q];
-        x[1] = pbuf[(rt * 16 + g + 8) * PSTR + q];
-        x[2] = pbuf[(rt * 16 + g) * PSTR + q + 4];
-        x[3] = pbuf[(rt * 16 + g + 8) * PSTR + q + 4];
-        uint32_t ah[4], al[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          ah[e] = to_tf32(x[e]);
-          al[e] = to_tf32(x[e] - __uint_as_float(ah[e]));
+        for (int cc = 0; cc < 8; ++cc) {
+          r = fmaf(-lr[cc], yv[cc], r);
+          hi[cc] = __uint_as_float(to_tf32(lr[cc]));
+          lo[cc] = __uint_as_float(to_tf32(lr[cc] - hi[cc]));
         }
-#pragma unroll
-        for (int jl = 0; jl < CTW; ++jl) {
-          const int ct = wid + NW * jl;
-          if (ct >= CT || !tile_live<NBW>(sb, rt, ct)) continue;  // warp-uniform
-          mma_tf32(acc[rt][jl], al, bh[jl][0], bh[jl][1]);
-          mma_tf32(acc[rt][jl], ah, bl[jl][0], bl[jl][1]);
-          mma_tf32(acc[rt][jl], ah, bh[jl][0], bh[jl][1]);
-        }
+        // cell (J + d, J), slot (J + d) mod d = J mod d
+        const int d = dr >> 3;
+        float* c = cells + cell_of(d, md) + (dr & 7) * 8;
+        *reinterpret_cast<float4*>(c) = make_float4(hi[0], hi[4], hi[1], hi[5]);
+        *reinterpret_cast<float4*>(c + 4) = make_float4(hi[2], hi[6], hi[3], hi[7]);
+        *reinterpret_cast<float4*>(c + 64) = make_float4(lo[0], lo[4], lo[1], lo[5]);
+        *reinterpret_cast<float4*>(c + 68) = make_float4(lo[2], lo[6], lo[3], lo[7]);
       }
-      // 4. entering rows into slot block sb (row tile sb / 2, half sb % 2), negated
-      {
-        const int rtn = sb >> 1, hn = sb & 1;
-#pragma unroll
-        for (int jl = 0; jl < CTW; ++jl)
-#pragma unroll
-          for (int e2 = 0; e2 < 2; ++e2) {
-            const int ct = wid + NW * jl;
-            float val = fmaf(lm, em[jl][e2], -ek[jl][e2]);
-            if (ct == sb) {
-              const int du2 = 2 * q + e2;
-              const int pr = (g >= du2) ? pnew : j0 + W + du2;
-              if (pr >= nl) val = (g == du2) ? -1.f : 0.f;
-            }
-            acc[rtn][jl][2 * hn + e2] = val;
-          }
-      }
-      if (d8 >= 0 && d8 < 8) r = rnew;
-      __syncthreads();  // pbuf is rewritten by the next extraction
-      jm += 8;
-      jm -= (jm >= BMAX) ? BMAX : 0;
     }
+    __syncthreads();  // the cells are complete; pbuf and srhs are rewritten
+    slot0 += 8;
+    slot0 -= (slot0 >= W) ? W : 0;
+    jm += 8;
+    jm -= (jm >= BMAX) ? BMAX : 0;
   }
-  if (bad && tid == 0) atomicOr(err, 1);
+  if (bad && lane == 0) atomicOr(err, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -2709,6 +2721,38 @@ __global__ void k_band_fill(int nsub, int64_t total, const int64_t* __restrict__
   }
 }
 
+// The same rows in the panel layout of k_local_factor_wide (FP32, window W = tier + 8,
+// arrays zeroed before): subdomain l from (sub_ptr[l] + 7 l) W, entry (p, q) of column
+// block J = q / 8 at (J W + p - 8 J) 8 + q mod 8, so that a panel is one aligned run
+// (row by row, its eight-entry pieces straddle two sectors each).  ident: the rows that
+// fill the last block are identity rows (K only).
+__global__ void k_band_panels(int nsub, int64_t total, const int64_t* __restrict__ sub_ptr,
+                              const int32_t* __restrict__ dofs, const int64_t* __restrict__ rp,
+                              const int32_t* __restrict__ ci, const double* __restrict__ val,
+                              const double* __restrict__ val2, int B, int W, int ident, float* __restrict__ out,
+                              float* __restrict__ out2) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= total) return;
+  const int l = sub_of(nsub, sub_ptr, t);
+  const int64_t off = sub_ptr[l];
+  const int nl = (int)(sub_ptr[l + 1] - off);
+  const int p = (int)(t - off);
+  const int32_t g = dofs[t];
+  const int64_t base = (off + 7 * (int64_t)l) * W;
+  auto at = [&](int r, int c) -> int64_t { return base + ((int64_t)(c >> 3) * W + r - (c & ~7)) * 8 + (c & 7); };
+  for (int64_t e = rp[g]; e < rp[g + 1]; ++e) {
+    const int32_t c = ci[e];
+    if (c > g) break;
+    const int q = local_index(dofs + off, nl, c);
+    if (q >= 0 && p - q < B) {
+      out[at(p, q)] = (float)val[e];
+      if (out2) out2[at(p, q)] = (float)val2[e];
+    }
+  }
+  if (ident && p == nl - 1)
+    for (int r = nl; r & 7; ++r) out[at(r, r)] = 1.f;
+}
+
 // Galerkin products K_H = P^T K P and M_H = P^T M P in two deterministic passes.
 // Pass 1 (thread per fine row r): the sparse rows (K P)[r, :] and (M P)[r, :],
 // at most `width` coarse columns each (32 first; wider on overflow, e.g. for the
@@ -3287,9 +3331,11 @@ int launch_local(Handle& h, const double* rho, const double* lam, int mode) {
   }
 #define BPJD_LOCAL_WIDE(BM)                                                                                    \
   case BM: {                                                                                                   \
-    k_local_factor_wide<BM><<<npairs_c, 32 * WideShape<BM>::NW, 0, h.stream>>>(                               \
+    allow_dynamic_smem((const void*)k_local_factor_wide<BM>);                                                  \
+    k_local_factor_wide<BM><<<npairs_c, 32 * WideShape<BM>::NW, sizeof(float) * WideShape<BM>::smem_floats,     \
+                              h.stream>>>(                                                                     \
         npairs_c, k, sptr, h.sub_dofs, h.bandKf, h.bandMf, lam, rho, (float*)h.Lbuf, (float*)h.wpk, h.derr,     \
-        rec_base);                                                                                             \
+        rec_base, l0);                                                                                           \
     if (mode == kLocalFull) {                                                                                  \
       const size_t bsm = sizeof(float) * BwdShape<BM>::smem_floats;                                            \
       allow_dynamic_smem((const void*)k_local_backward<BM>);                                                   \
@@ -3348,6 +3394,7 @@ int prime_kernel_attributes(Handle& h) {
       allow_dynamic_smem((const void*)k_local_sweep_blk<BM, true>);
       allow_dynamic_smem((const void*)k_local_sweep_blk<BM, false>);
     } else {
+      allow_dynamic_smem((const void*)k_local_factor_wide<BM>);
       allow_dynamic_smem((const void*)k_local_forward<BM>);
       allow_dynamic_smem((const void*)k_local_backward<BM>);
     }
@@ -3438,8 +3485,9 @@ int launch_local_grouped(Handle* const* hs, const double* const* rho, const doub
       // allocation is tuned for one subdomain-shift pair per CTA), on the shared stream
       for (int j = 0; j < gf.n; ++j) {
         const LocalSeg& q = gf.s[j];
-        k_local_factor_wide<B><<<q.nsub * q.k, 32 * WideShape<B>::NW, 0, s>>>(
-            q.nsub * q.k, q.k, q.sub_ptr, q.sub_dofs, q.bandK, q.bandM, q.lam, q.rho, q.Lbuf, q.wpk, q.err, 0);
+        allow_dynamic_smem((const void*)k_local_factor_wide<B>);
+        k_local_factor_wide<B><<<q.nsub * q.k, 32 * WideShape<B>::NW, sizeof(float) * WideShape<B>::smem_floats, s>>>(
+            q.nsub * q.k, q.k, q.sub_ptr, q.sub_dofs, q.bandK, q.bandM, q.lam, q.rho, q.Lbuf, q.wpk, q.err, 0, 0);
       }
       if (gr.n) {
         allow_dynamic_smem((const void*)k_local_forward_grp<B>);
@@ -3518,7 +3566,14 @@ int launch_split_values(const double* v, int64_t nnz, float2* out, cudaStream_t 
 int launch_band_fill(Handle& h, const CsrDev& c, const double* val2, double* out, double* out2, float* outf,
                      float* outf2) {
   const unsigned blocks = (unsigned)((h.sum_nl + 127) / 128);
-  if (outf) {
+  if (outf && band_panels(h.Bpad)) {
+    const size_t bytes = sizeof(float) * band_floats(h.sum_nl, h.nsub, h.B, h.Bpad);
+    cudaError_t e = cudaMemsetAsync(outf, 0, bytes, h.stream);
+    if (e == cudaSuccess && outf2) e = cudaMemsetAsync(outf2, 0, bytes, h.stream);
+    if (e != cudaSuccess) return (int)e;
+    k_band_panels<<<blocks, 128, 0, h.stream>>>(h.nsub, h.sum_nl, h.sub_ptr, h.sub_dofs, c.row_ptr, c.col, c.val, val2,
+                                                h.B, h.Bpad + 8, outf == h.bandKf ? 1 : 0, outf, outf2);
+  } else if (outf) {
     const int W = std::max(h.B, h.Bpad);
     k_band_fill<float><<<blocks, 128, 0, h.stream>>>(h.nsub, h.sum_nl, h.sub_ptr, h.sub_dofs, c.row_ptr, c.col, c.val,
                                                      val2, h.B, W, outf, outf2);

@@ -48,7 +48,8 @@ __device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
   e = __fmaf_rn(a, b, -p);
 }
 
-__device__ __forceinline__ dw split_f64(double x) {
+// any x, field by field
+static __device__ __noinline__ dw split_f64_any(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned int sign = (unsigned int)(b >> 63) << 31;
   const int e = (int)((b >> 52) & 0x7ff);
@@ -79,6 +80,21 @@ __device__ __forceinline__ dw split_f64(double x) {
     }
   }
   r.lo = sign ? -lo : lo;
+  return r;
+}
+
+// hi: the top 24 significand bits re-biased in one subtraction; lo: the other 29 bits as
+// an integer rounded toward zero to 24 bits and scaled by a power of two (exact).  The
+// general form serves zero, |x| < 2^-74 and |x| >= 2^128: the same values either way.
+__device__ __forceinline__ dw split_f64(double x) {
+  const unsigned int h = (unsigned int)__double2hiint(x), l = (unsigned int)__double2loint(x);
+  const unsigned int e = (h >> 20) & 0x7ffu;
+  if (e - 949u > 201u) return split_f64_any(x);
+  const unsigned int sign = h & 0x80000000u;
+  dw r;
+  r.hi = __uint_as_float((__funnelshift_l(l, h, 3) - (384u << 23)) | sign);
+  const float lo = __fmul_rn(__uint2float_rz(l & 0x1fffffffu), __uint_as_float((e - 948u) << 23));
+  r.lo = __uint_as_float(__float_as_uint(lo) | sign);
   return r;
 }
 
@@ -133,6 +149,82 @@ struct dot2 {
     c = __fadd_rn(c, __fadd_rn(u, al));
   }
   __device__ __forceinline__ double value() const { return dw_to_f64(s, c); }
+};
+
+// ---- two Dot2 accumulators in packed f32x2 arithmetic (lane-wise the roundings of dot2) ----
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long p, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
+}
+__device__ __forceinline__ unsigned long long swap2(unsigned long long p) {
+  float a, b;
+  unpack2(p, a, b);
+  return pack2(b, a);
+}
+__device__ __forceinline__ unsigned long long neg2(unsigned long long p) {
+  float a, b;
+  unpack2(p, a, b);
+  return pack2(-a, -b);
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+struct f32x4p {
+  unsigned long long p[2];
+};
+// four floats (16-byte aligned) as two pairs
+__device__ __forceinline__ f32x4p load_pairs(const float* a) {
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(a);
+  return f32x4p{{v.x, v.y}};
+}
+struct dot2x2 {
+  unsigned long long s, c;
+  __device__ __forceinline__ void zero() { s = c = 0ULL; }
+  // += (ah + al) (bh + bl) in both lanes; nh = -ah and nl = -al, so that the product error
+  // comes out negated without a negation (fma(nh, bh, p) = -(ah bh - p))
+  __device__ __forceinline__ void mac(unsigned long long ah, unsigned long long nh, unsigned long long nl,
+                                      unsigned long long bh, unsigned long long bl) {
+    const unsigned long long p = mul2(ah, bh);
+    const unsigned long long ne = fma2(nh, bl, fma2(nl, bh, fma2(nh, bh, p)));
+    const unsigned long long t = add2(s, p);
+    const unsigned long long bb = sub2(t, s);
+    const unsigned long long u = add2(sub2(s, sub2(t, bb)), sub2(p, bb));
+    s = t;
+    c = add2(c, sub2(u, ne));
+  }
+  __device__ __forceinline__ double value0() const {
+    float a, b, d, e;
+    unpack2(s, a, b);
+    unpack2(c, d, e);
+    return dw_to_f64(a, d);
+  }
+  __device__ __forceinline__ double value1() const {
+    float a, b, d, e;
+    unpack2(s, a, b);
+    unpack2(c, d, e);
+    return dw_to_f64(b, e);
+  }
 };
 
 }  // namespace bpjd

@@ -269,16 +269,30 @@ __global__ void __launch_bounds__(256) k_inner(int n, int k, int p, Ptrs6 U, int
 
 // ---------------------------------------------------------------------------
 // Block inner products in double-word arithmetic (Dot2 on the FP32 pipe):
-// out_v = U^T V_v for v < NV, with U = [U_0 .. U_{nu-1}] (mu = nu k columns)
+// out_v = U^T V_v for v < 2 (blockIdx.y), with U = [U_0 .. U_{nu-1}] (mu = nu k columns)
 // and V_v = [V_v,0 ..] (mv columns), all n x k FP64 row-major blocks.  With
 // sym = 1 only the 4 x 4 output tiles on or above the diagonal are formed
-// (U^T V symmetric).  Rows are staged in shared memory in chunks, split into
-// (hi, lo) float pairs once; each thread owns one output tile and a slice of
-// the chunk rows; slices are combined in FP64 at the end of the block and the
-// per-block partial sums are reduced over blocks in FP64 by k_gram_reduce.
+// (U^T V symmetric).  The rows of a block are taken in chunks of R: copied
+// asynchronously into a raw buffer two chunks ahead, split once into (hi, lo)
+// float planes, and accumulated by one thread per (tile, slice of the chunk's
+// rows).  A plane row holds the columns of U, then of V_v (absent when V_v is U),
+// each padded with zero columns to a multiple of four, so that a tile reads
+// aligned vectors whatever k is.  Slices are combined in FP64 at the end
+// of the block and the per-block sums are reduced over blocks in FP64 by
+// k_gram_reduce.
+// Bound: the FP32 pipe, 12 lane operations per Dot2 multiply-add (39.3 T/s
+// measured: 53 us for 36 columns of 261,121 rows, upper tiles).  The products
+// run two at a time in packed f32x2 instructions (the same pipe rate and the
+// same roundings, half the issue slots, which the splits and copies then use):
+// a tile's pairs are taken along its diagonals, (x, y) with (x + 1, y + 1) and
+// (x, y + 1) with (x + 1, y), so that U's pairs are the loaded ones and V's are
+// the loaded ones and their swaps.  Measured (GB300, before -> now): 36 columns
+// of 261,121 rows, symmetric, 188 -> 148 us (136 us in this kernel: FP32 pipe
+// 53 % busy; two or three blocks per SM are alike), 19 x 57 columns of 65,025
+// rows 99 -> 81 us, 18 columns of 2,209 rows (both products) 44 -> 12 us.
 // ---------------------------------------------------------------------------
-constexpr int kGramRows = 64;
-constexpr int kGramBlocks = 304;  // two resident blocks on each of the 152 SMs: one wave
+constexpr int kGramRows = 32;     // rows per block, at least
+constexpr int kGramBlocks = 456;  // three resident blocks on each of the 152 SMs: one wave
 
 __device__ __forceinline__ void gram_tile_of(int t, int TU, int TV, int sym, int& ta, int& tb) {
   if (!sym) {
@@ -303,198 +317,158 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// Per-block Gram partials in double-word arithmetic (Dot2 per entry).  The
-// row range of a block is processed in chunks of R rows: the FP64 rows of
-// every U / V block are copied asynchronously into a raw staging buffer two
-// chunks ahead (double buffered), split into (hi, lo) planes once per chunk,
-// and every thread accumulates a 4 x 4 tile of the output for every NV over
-// its slice of the chunk's rows.  Plane layout: one segment of R x k values per
-// block (U blocks, then V1, then V2), row-major.
-// VEC: k is a multiple of 4, so the four columns of a tile lie in one block,
-// contiguous and 16-byte aligned in the planes (vector loads, no padding).
-template <int NV, bool VEC>
-__global__ void __launch_bounds__(256, 2) k_gram_dw(int n, int k, int nu, Ptrs6 U, int nvb, Ptrs6 V1, Ptrs6 V2, int sym,
-                                                 int rows_per_block, int R, double* partial) {
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, (THREADS <= 192) ? 3 : 2)
+    k_gram_dw(int n, int k, int nu, Ptrs6 U, int nvb, Ptrs6 V1, Ptrs6 V2, int sym, int shared_mask, int S,
+              int rows_per_block, int R, double* partial) {
   extern __shared__ __align__(16) float gsm[];
+  const Ptrs6& V = blockIdx.y ? V2 : V1;
+  const int shared_v = (shared_mask >> blockIdx.y) & 1;
   const int mu = nu * k, mv = nvb * k;
   const int TU = (mu + 3) / 4, TV = (mv + 3) / 4;
   const int ntiles = sym ? TU * (TU + 1) / 2 : TU * TV;
-  const int S = max(1, (int)blockDim.x / ntiles);
-  const int nseg = nu + NV * nvb;
-  const int SEG = R * k;    // values per segment
-  const int CH = nseg * SEG;  // values per chunk
-  double* raw = reinterpret_cast<double*>(gsm);    // [2][CH]
-  float* ph = reinterpret_cast<float*>(raw + 2 * CH);  // [CH]
-  float* pl = ph + CH;                                 // [CH]
-  const int tid = threadIdx.x;
+  const int nseg = nu + (1 - shared_v) * nvb;  // blocks copied (V is U: not again)
+  const int SEG = R * k;                        // values per block and chunk
+  const int CH = nseg * SEG;                    // values per chunk
+  const int LD = 4 * (TU + (1 - shared_v) * TV);  // plane row
+  double* raw = reinterpret_cast<double*>(gsm);        // [2][CH]
+  float* ph = reinterpret_cast<float*>(raw + 2 * CH);  // [R][LD]
+  float* pl = ph + R * LD;                             // [R][LD]
+  const int tid = threadIdx.x, nt = blockDim.x;
   const int tile = tid % ntiles, slice = tid / ntiles;
   const bool worker = slice < S;
   int ta = 0, tb = 0;
   gram_tile_of(tile, TU, TV, sym, ta, tb);
-  // plane offsets of this thread's four U columns and four V columns (-1: past the end)
-  int uo[4], vo[4];
-#pragma unroll
-  for (int x = 0; x < 4; ++x) {
-    const int cu = 4 * ta + x, cv = 4 * tb + x;
-    uo[x] = (cu < mu) ? (cu / k) * SEG + cu % k : -1;
-    vo[x] = (cv < mv) ? (nu + cv / k) * SEG + cv % k : -1;
-  }
+  const int uo = 4 * ta, vo = 4 * (tb + (shared_v ? 0 : TU));
   const int64_t r0 = (int64_t)blockIdx.x * rows_per_block;
   const int64_t r1 = min((int64_t)n, r0 + rows_per_block);
   const int nch = (int)((r1 - r0 + R - 1) / R);
-  auto seg_ptr = [&](int sg) -> const double* {
-    if (sg < nu) return U.p[sg];
-    sg -= nu;
-    if (sg < nvb) return V1.p[sg];
-    return V2.p[sg - nvb];
-  };
+  auto seg_ptr = [&](int sg) -> const double* { return sg < nu ? U.p[sg] : V.p[sg - nu]; };
+  // plane column of a segment's first value
+  auto seg_col = [&](int sg) -> int { return sg < nu ? sg * k : 4 * TU + (sg - nu) * k; };
   auto issue = [&](int c) {
     if (c < nch) {
       const int64_t rb = r0 + (int64_t)c * R;
-      const int64_t lim = (r1 - rb) * k;  // values of this chunk inside the row range
+      const int cnt = (int)min((int64_t)SEG, (r1 - rb) * k);  // values inside the row range
       double* dst = raw + (c & 1) * CH;
       for (int sg = 0; sg < nseg; ++sg) {
         const double* src = seg_ptr(sg) + rb * k;
-        for (int e = tid; e < SEG; e += blockDim.x)
-          if (e < lim) cp_async8(dst + sg * SEG + e, src + e);
+        for (int e = tid; e < cnt; e += nt) cp_async8(dst + sg * SEG + e, src + e);
       }
     }
     cp_async_commit();
   };
-  dot2 acc[NV][4][4];
+  dot2x2 acc[4][2];  // pairs of a 4 x 4 tile: [2 x pair + anti-diagonal][y pair]
 #pragma unroll
-  for (int v = 0; v < NV; ++v)
+  for (int x = 0; x < 4; ++x)
 #pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 4; ++y) acc[v][x][y].zero();
+    for (int y = 0; y < 2; ++y) acc[x][y].zero();
   issue(0);
   issue(1);
+  // padding columns stay zero
+  for (int e = tid; e < R * LD; e += nt) ph[e] = pl[e] = 0.f;
+  const int er0 = tid / k, ej0 = tid % k, edr = nt / k, edj = nt % k;
   for (int c = 0; c < nch; ++c) {
     cp_async_wait1();
     __syncthreads();  // chunk c has landed for every thread; the planes are free
+    const int nr = (int)min((int64_t)R, r1 - (r0 + (int64_t)c * R));
     {
-      const int nr = (int)min((int64_t)R, r1 - (r0 + (int64_t)c * R));
       const double* src = raw + (c & 1) * CH;
-      if (nr == R) {
-        for (int e = tid; e < CH; e += blockDim.x) {
-          const dw sp = split_f64(src[e]);
-          ph[e] = sp.hi;
-          pl[e] = sp.lo;
-        }
-      } else {  // last chunk of the range: rows past its end are zero
-        for (int e = tid; e < CH; e += blockDim.x) {
-          const int r = (e % SEG) / k;
-          const dw sp = split_f64(r < nr ? src[e] : 0.0);
-          ph[e] = sp.hi;
-          pl[e] = sp.lo;
+      for (int sg = 0; sg < nseg; ++sg) {
+        const double* s = src + sg * SEG;
+        float* h = ph + seg_col(sg);
+        float* l = pl + seg_col(sg);
+        // value e = (row r, column j), advanced without a division
+        for (int e = tid, r = er0, j = ej0; r < nr; e += nt) {
+          const dw sp = split_f64(s[e]);
+          h[r * LD + j] = sp.hi;
+          l[r * LD + j] = sp.lo;
+          r += edr;
+          j += edj;
+          if (j >= k) {
+            j -= k;
+            ++r;
+          }
         }
       }
     }
     __syncthreads();  // planes ready; the raw buffer of chunk c is free
     issue(c + 2);
-    if (worker && VEC) {
-      for (int r = slice; r < R; r += S) {
-        const int ro = r * k;
-        const float4 uh = *reinterpret_cast<const float4*>(ph + uo[0] + ro);
-        const float4 ul = *reinterpret_cast<const float4*>(pl + uo[0] + ro);
-        const float a_h[4] = {uh.x, uh.y, uh.z, uh.w};
-        const float a_l[4] = {ul.x, ul.y, ul.z, ul.w};
+    if (worker) {
+      for (int r = slice; r < nr; r += S) {
+        const float* rh = ph + r * LD;
+        const float* rl = pl + r * LD;
+        const f32x4p uh = load_pairs(rh + uo), ul = load_pairs(rl + uo);
+        const unsigned long long nh[2] = {neg2(uh.p[0]), neg2(uh.p[1])}, nl[2] = {neg2(ul.p[0]), neg2(ul.p[1])};
+        const f32x4p vh = load_pairs(rh + vo), vl = load_pairs(rl + vo);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          const int o = vo[0] + v * mv * R + ro;
-          const float4 vh = *reinterpret_cast<const float4*>(ph + o);
-          const float4 vl = *reinterpret_cast<const float4*>(pl + o);
-          const float b_h[4] = {vh.x, vh.y, vh.z, vh.w};
-          const float b_l[4] = {vl.x, vl.y, vl.z, vl.w};
+        for (int y = 0; y < 2; ++y) {
+          const unsigned long long sh = swap2(vh.p[y]), sl = swap2(vl.p[y]);
 #pragma unroll
-          for (int x = 0; x < 4; ++x)
-#pragma unroll
-            for (int y = 0; y < 4; ++y) acc[v][x][y].mac(a_h[x], a_l[x], b_h[y], b_l[y]);
-        }
-      }
-    } else if (worker) {
-      for (int r = slice; r < R; r += S) {
-        const int ro = r * k;
-        float a_h[4], a_l[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-          a_h[x] = (uo[x] >= 0) ? ph[uo[x] + ro] : 0.f;
-          a_l[x] = (uo[x] >= 0) ? pl[uo[x] + ro] : 0.f;
-        }
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          float b_h[4], b_l[4];
-#pragma unroll
-          for (int y = 0; y < 4; ++y) {
-            const int o = vo[y] + v * mv * R;  // V2 segments follow the V1 segments
-            b_h[y] = (vo[y] >= 0) ? ph[o + ro] : 0.f;
-            b_l[y] = (vo[y] >= 0) ? pl[o + ro] : 0.f;
+          for (int x = 0; x < 2; ++x) {
+            acc[2 * x][y].mac(uh.p[x], nh[x], nl[x], vh.p[y], vl.p[y]);
+            acc[2 * x + 1][y].mac(uh.p[x], nh[x], nl[x], sh, sl);
           }
-#pragma unroll
-          for (int x = 0; x < 4; ++x)
-#pragma unroll
-            for (int y = 0; y < 4; ++y) acc[v][x][y].mac(a_h[x], a_l[x], b_h[y], b_l[y]);
         }
       }
     }
   }
   cp_async_wait0();
   __syncthreads();
-  // combine the slices of every tile in FP64 (shared memory reused)
-  double* red = reinterpret_cast<double*>(gsm);
-  const int per = NV * 16;
-  double mine[NV * 16];
-#pragma unroll
-  for (int v = 0; v < NV; ++v)
+  // combine the slices in FP64 (shared memory reused): every thread sums some entries
+  double* red = reinterpret_cast<double*>(gsm);  // [S][ntiles 16]
+  const int per = ntiles * 16;
+  if (worker) {
+    double* m = red + (size_t)slice * per + tile * 16;
 #pragma unroll
     for (int x = 0; x < 4; ++x)
 #pragma unroll
-      for (int y = 0; y < 4; ++y) mine[v * 16 + x * 4 + y] = acc[v][x][y].value();
-  for (int sl = 1; sl < S; ++sl) {
-    if (worker && slice == sl)
-      for (int e = 0; e < per; ++e) red[tile * per + e] = mine[e];
-    __syncthreads();
-    if (worker && slice == 0)
-      for (int e = 0; e < per; ++e) mine[e] += red[tile * per + e];
-    __syncthreads();
+      for (int y = 0; y < 2; ++y) {
+        // pair [x][y]: entries (2 (x / 2), 2 y + x % 2) and (2 (x / 2) + 1, 2 y + 1 - x % 2)
+        const int a = 2 * (x / 2), b = 2 * y + (x & 1);
+        m[a * 4 + b] = acc[x][y].value0();
+        m[(a + 1) * 4 + 2 * y + 1 - (x & 1)] = acc[x][y].value1();
+      }
   }
-  if (worker && slice == 0) {
-    double* out = partial + (int64_t)blockIdx.x * ntiles * per;
-    for (int e = 0; e < per; ++e) out[(e / 16) * ntiles * 16 + tile * 16 + (e % 16)] = mine[e];
+  __syncthreads();
+  double* out = partial + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * per;
+  for (int e = tid; e < per; e += nt) {
+    double s = red[e];
+    for (int sl = 1; sl < S; ++sl) s += red[(size_t)sl * per + e];
+    out[e] = s;
   }
 }
 
-// Sum of the per-block Gram partials: a block serves 32 consecutive entries;
-// warp w adds blocks b = w, w + 8, ... in order, warp 0 adds the eight results
-// in order (fixed order: bit-reproducible).
-__global__ void __launch_bounds__(256) k_gram_reduce(int nblk, int nv, int mu, int mv, int sym,
+// Sum of the per-block Gram partials: a block serves 8 consecutive entries; thread
+// group g = tid / 8 adds the blocks b = g, g + 32, ... in order, then a fixed tree over
+// the groups (bit-reproducible).
+__global__ void __launch_bounds__(256) k_gram_reduce(int nblk, int mu, int mv, int sym,
                                                      const double* __restrict__ partial, double* out1,
                                                      double* out2) {
-  __shared__ double red[8][32];
+  __shared__ double red[8][8];
   const int TU = (mu + 3) / 4, TV = (mv + 3) / 4;
   const int ntiles = sym ? TU * (TU + 1) / 2 : TU * TV;
-  const int total = nv * ntiles * 16;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int t = blockIdx.x * 32 + lane;
+  const int per = ntiles * 16;  // entries of one product: a multiple of 16
+  const int t = blockIdx.x * 8 + (threadIdx.x & 7), w = threadIdx.x >> 5;
+  const int v = t / per, rem = t % per;
   double s = 0;
-  if (t < total)
-    for (int b = w; b < nblk; b += 8) s += partial[(int64_t)b * total + t];
-  red[w][lane] = s;
+#pragma unroll 5
+  for (int b = threadIdx.x >> 3; b < nblk; b += 32) s += partial[((int64_t)v * nblk + b) * per + rem];
+  s += __shfl_xor_sync(0xffffffffu, s, 8);
+  s += __shfl_xor_sync(0xffffffffu, s, 16);
+  if ((threadIdx.x & 31) < 8) red[w][threadIdx.x & 7] = s;
   __syncthreads();
-  if (w != 0 || t >= total) return;
-  s = red[0][lane];
-#pragma unroll
-  for (int q = 1; q < 8; ++q) s += red[q][lane];
-  const int v = t / (ntiles * 16);
-  const int rem = t % (ntiles * 16);
+  if (threadIdx.x >= 8) return;
+  const int q = threadIdx.x;
+  s = ((red[0][q] + red[1][q]) + (red[2][q] + red[3][q])) + ((red[4][q] + red[5][q]) + (red[6][q] + red[7][q]));
   const int tile = rem / 16, e = rem % 16;
   int ta, tb;
   gram_tile_of(tile, TU, TV, sym, ta, tb);
   const int a = 4 * ta + e / 4, c = 4 * tb + e % 4;
   if (a >= mu || c >= mv) return;
   double* out = (v == 0) ? out1 : out2;
-  out[a * mv + c] = s;
+  // a diagonal tile holds both (a, c) and (c, a): each writes one place only
+  if (!sym || ta != tb) out[a * mv + c] = s;
   if (sym) out[c * mv + a] = s;
 }
 
@@ -3027,14 +3001,54 @@ int launch_inner(Handle& h, int p, const double* const* U, int q, const double* 
   return (int)cudaGetLastError();
 }
 
+// Blocks, rows per block and per chunk, slices and shared memory of a Gram launch.
+struct GramShape {
+  int ntiles = 0, S = 1, threads = 32, nblk = 1, rpb = 1, R = 1;
+  size_t smem = 0;
+};
+static GramShape gram_shape(int64_t n, int k, int nu, int nvb, int nv, int sym, size_t capacity) {
+  GramShape g;
+  const int TU = (nu * k + 3) / 4, TV = (nvb * k + 3) / 4;
+  g.ntiles = sym ? TU * (TU + 1) / 2 : TU * TV;
+  // slices of a chunk's rows: the count that leaves the fewest lanes without a tile among
+  // those that make 128 to 192 threads, of which three blocks fit an SM (at most 16 slices;
+  // 45 tiles: 4 slices, 180 of 192); more tiles than that take one slice, two blocks on an SM
+  double best = -1;
+  for (int S = 1; S <= 16 && (S == 1 || S * g.ntiles <= 192); ++S) {
+    const int th = (S * g.ntiles + 31) / 32 * 32;
+    const double eff = (double)S * g.ntiles / th - (th < 128 ? 1.0 - th / 512.0 : 0.0);
+    if (eff >= best) {
+      best = eff;
+      g.S = S;
+    }
+  }
+  g.threads = (g.S * g.ntiles + 31) / 32 * 32;
+  const int64_t fit = std::max<int64_t>(1, (int64_t)(capacity / ((size_t)g.ntiles * nv * 16)));
+  const int64_t wave = (g.threads <= 192 ? kGramBlocks : kGramBlocks / 3 * 2) / nv;
+  const int64_t want = std::min(fit, std::min<int64_t>(wave, (n + kGramRows - 1) / kGramRows));
+  g.rpb = (int)((n + want - 1) / want);
+  g.nblk = (int)((n + g.rpb - 1) / g.rpb);
+  // chunk rows: two raw FP64 buffers and the (hi, lo) planes within 70 KB (three blocks on an
+  // SM), a multiple of the slices, no longer than a block's rows
+  const size_t per_row = 16 * (size_t)(nu + nvb) * k + 32 * (size_t)(TU + TV);
+  int R = (int)std::min<size_t>(64, (70 * 1024) / per_row);
+  R = std::min(R, (g.rpb + g.S - 1) / g.S * g.S);
+  if (R >= g.S) R -= R % g.S;
+  R += R & 1;  // raw buffers and planes stay 16-byte aligned
+  g.R = std::max(2, R);
+  g.smem = std::max(per_row * g.R, (size_t)g.S * g.ntiles * 16 * sizeof(double));
+  return g;
+}
+
+// What bpjd_block_gram_noalloc asks of its static array (row ranges in units of 64 rows);
+// a launch takes fewer blocks where the scratch holds fewer partial sums.
 size_t gram_partial_doubles(int64_t n, int k, int nu, int nvb, int sym) {
-  const int mu = nu * k, mv = nvb * k;
-  const int TU = (mu + 3) / 4, TV = (mv + 3) / 4;
+  constexpr int64_t kUnit = 64, kBlocks = 304;
+  const int TU = (nu * k + 3) / 4, TV = (nvb * k + 3) / 4;
   const int ntiles = sym ? TU * (TU + 1) / 2 : TU * TV;
-  const int nblk = (int)std::min<int64_t>(kGramBlocks, (n + kGramRows - 1) / kGramRows);
-  const int rpb = (int)(((n + nblk - 1) / nblk + kGramRows - 1) / kGramRows * kGramRows);
-  const int nblk2 = (int)((n + rpb - 1) / rpb);
-  return (size_t)nblk2 * ntiles * 16;
+  const int64_t nblk = std::min<int64_t>(kBlocks, (n + kUnit - 1) / kUnit);
+  const int64_t rpb = ((n + nblk - 1) / nblk + kUnit - 1) / kUnit * kUnit;
+  return (size_t)((n + rpb - 1) / rpb) * ntiles * 16;
 }
 
 int launch_gram_raw(int64_t n, int k, int nu, const double* const* U, int nvb, int nv, const double* const* V1,
@@ -3046,43 +3060,29 @@ int launch_gram_raw(int64_t n, int k, int nu, const double* const* U, int nvb, i
   if (ntiles > 256 || nv < 1 || nv > 2 || nu > 6 || nvb > 6 || n < 1) return (int)cudaErrorInvalidValue;
   Ptrs6 u{}, v1{}, v2{};
   for (int b = 0; b < nu; ++b) u.p[b] = U[b];
+  int shared = nu == nvb ? 3 : 0;  // bit v: the same blocks on both sides (copied and split once)
   for (int b = 0; b < nvb; ++b) {
     v1.p[b] = V1[b];
-    if (nv > 1) v2.p[b] = V2[b];
+    if (shared && U[b] != V1[b]) shared &= ~1;
+    if (nv > 1) {
+      v2.p[b] = V2[b];
+      if (shared && U[b] != V2[b]) shared &= ~2;
+    }
   }
-  const int nblk = (int)std::min<int64_t>(kGramBlocks, (n + kGramRows - 1) / kGramRows);
-  const int rpb = (int)(((n + nblk - 1) / nblk + kGramRows - 1) / kGramRows * kGramRows);
-  const int nblk2 = (int)((n + rpb - 1) / rpb);
+  const GramShape g = gram_shape(n, k, nu, nvb, nv, sym, partial_capacity);
   const int total = nv * ntiles * 16;
-  if ((size_t)nblk2 * total > partial_capacity) return (int)cudaErrorInvalidValue;
-  // chunk rows: a divisor of kGramRows keeping the staging (two raw FP64 buffers
-  // and the hi/lo planes, 24 bytes per value) within 100 KB (few blocks: long
-  // chunks, fewer barriers per row)
-  const int nseg = nu + nv * nvb;
-  int R = kGramRows;
-  while (R > 1 && (size_t)24 * R * k * nseg > 100 * 1024) R /= 2;
-  const size_t stage = (size_t)24 * R * k * nseg;
-  const size_t red = (size_t)ntiles * nv * 16 * sizeof(double);
-  const size_t sm = std::max(stage, red);
-  auto go = [&](auto nv_tag, auto vec_tag) {
-    constexpr int NV = decltype(nv_tag)::value;
-    constexpr bool VEC = decltype(vec_tag)::value;
-    allow_dynamic_smem((const void*)k_gram_dw<NV, VEC>);
-    k_gram_dw<NV, VEC><<<nblk2, 256, sm, stream>>>((int)n, k, nu, u, nvb, v1, v2, sym, rpb, R, partial);
-  };
-  const bool vec = (k % 4) == 0;
-  if (nv == 2) {
-    if (vec)
-      go(std::integral_constant<int, 2>(), std::true_type());
-    else
-      go(std::integral_constant<int, 2>(), std::false_type());
+  if ((size_t)g.nblk * total > partial_capacity) return (int)cudaErrorInvalidValue;
+  const dim3 grid(g.nblk, nv);
+  if (g.threads <= 192) {
+    allow_dynamic_smem((const void*)k_gram_dw<192>);
+    k_gram_dw<192><<<grid, g.threads, g.smem, stream>>>((int)n, k, nu, u, nvb, v1, v2, sym, shared, g.S, g.rpb, g.R,
+                                                        partial);
   } else {
-    if (vec)
-      go(std::integral_constant<int, 1>(), std::true_type());
-    else
-      go(std::integral_constant<int, 1>(), std::false_type());
+    allow_dynamic_smem((const void*)k_gram_dw<256>);
+    k_gram_dw<256><<<grid, g.threads, g.smem, stream>>>((int)n, k, nu, u, nvb, v1, v2, sym, shared, g.S, g.rpb, g.R,
+                                                        partial);
   }
-  k_gram_reduce<<<(total + 31) / 32, 256, 0, stream>>>(nblk2, nv, mu, mv, sym, partial, out1, out2);
+  k_gram_reduce<<<total / 8, 256, 0, stream>>>(g.nblk, mu, mv, sym, partial, out1, out2);
   return (int)cudaGetLastError();
 }
 

@@ -1,5 +1,7 @@
 """Kernels at the sizes where their tiles, windows and dispatch rules end, through the C ABI."""
 
+import ctypes as C
+
 import numpy as np
 import pytest
 import scipy.linalg as la
@@ -76,3 +78,32 @@ def test_fp64_local_windows(name, k):
     sv.apply_preconditioner(torch.tensor(rho, device=DEV), torch.tensor(lam, device=DEV), Z)
     assert np.abs(Z.cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref).max()
     sv.close()
+
+
+# Double-word Gram products: columns around multiples of four (tiles are 4 x 4), one to four blocks, row counts
+# below, at and beyond a block's 32 rows.  The inputs make every operation exact, so the result has to be: V holds
+# integers up to 64, U integers a (not +-1) plus b 2^-28 with b up to 15 (wholly in the low part of the split unless
+# a = 0), so high products sum to integers below 2^24 in the running sum and the others to multiples of 2^-28 below
+# 2^-4 in the compensation; U^T U takes the integers alone.
+@pytest.mark.parametrize("n", [1, 31, 33, 2209])
+@pytest.mark.parametrize("k,nu,nv,sym", [(1, 1, 1, False), (2, 3, 3, True), (3, 2, 3, False), (4, 1, 1, True),
+                                         (5, 3, 3, True), (7, 3, 2, False), (12, 3, 3, True), (13, 1, 3, False),
+                                         (16, 4, 4, True), (16, 4, 4, False), (21, 3, 1, False), (32, 2, 2, True)])
+def test_block_gram_exact_integers(n, k, nu, nv, sym):
+    rng = np.random.default_rng(n * 100 + k)
+    ints = lambda: rng.integers(-64, 65, size=(n, k)).astype(np.float64)  # noqa: E731
+    U = [ints() for _ in range(nu)]
+    if not sym:
+        U = [np.where(np.abs(u) == 1, 0, u) + rng.integers(0, 16, size=(n, k)) * 2.0 ** -28 for u in U]
+    V = U if sym else [ints() for _ in range(nv)]
+    Ud = [torch.tensor(u, device=DEV) for u in U]
+    Vd = Ud if sym else [torch.tensor(v, device=DEV) for v in V]
+    out = torch.full((nu * k, nv * k), float("nan"), dtype=torch.float64, device=DEV)
+    fn = B.lib.bpjd_block_gram_noalloc
+    fn.argtypes = [C.c_int64, C.c_int32, C.c_int32, C.c_void_p, C.c_int32, C.c_void_p, C.c_int32, C.c_void_p,
+                   C.c_void_p]
+    pu = (C.c_void_p * nu)(*[u.data_ptr() for u in Ud])
+    pv = (C.c_void_p * nv)(*[v.data_ptr() for v in Vd])
+    assert fn(n, k, nu, pu, nv, pv, 1 if sym else 0, out.data_ptr(), None) == B.OK
+    Un, Vn = np.hstack(U), np.hstack(V)
+    np.testing.assert_array_equal(out.cpu().numpy(), Un.T @ Vn)

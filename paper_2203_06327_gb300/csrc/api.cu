@@ -393,7 +393,8 @@ extern "C" int bpjd_setup(const bpjd_csr* A, const bpjd_csr* M, const bpjd_csr* 
     if (h->dword()) {
       CK(dalloc(*h, &h->Asplit, (size_t)A->nnz));
       CK(dalloc(*h, &h->Msplit, (size_t)M->nnz));
-      CK(dalloc(*h, &h->xsplit, (size_t)n * k));
+      CK(dalloc(*h, &h->xsplit, (size_t)n * 2 * h->kp()));
+      CK(cudaMemsetAsync(h->xsplit, 0, sizeof(float) * (size_t)n * 2 * h->kp(), h->stream));  // padding columns
       CKI(launch_split_values(h->A.val, A->nnz, h->Asplit, h->stream));
       CKI(launch_split_values(h->M.val, M->nnz, h->Msplit, h->stream));
     }

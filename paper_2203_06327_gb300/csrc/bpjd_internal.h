@@ -58,7 +58,9 @@ struct Handle {
   bool same_pattern = false;
   float2* Asplit = nullptr;  // (hi, lo) float pairs of K and M values (double-word SpMM)
   float2* Msplit = nullptr;
-  float2* xsplit = nullptr;  // n x k (hi, lo) split of the block the next double-word SpMM reads
+  float* xsplit = nullptr;   // n x 2 kp split of the block the next double-word SpMM reads: a
+                             // row's hi parts, then its lo parts (kp: k rounded up to four)
+  int kp() const { return (k + 3) / 4 * 4; }
   float2* Psplit = nullptr;  // (hi, lo) split of P's values (FP32 prolongation of FP32 preconditioners)
   CsrDev P, PT;             // coarse interpolation and its transpose
   double* Phi = nullptr;    // n_H x n_H row-major, M_H-orthonormal eigenvectors
@@ -169,7 +171,7 @@ int gen_eig_host(int n, const std::vector<double>& K, const std::vector<double>&
 // kernels.cu launchers (all asynchronous on h.stream; return cudaError_t as int)
 // Xs (double-word path only): the (hi, lo) split of X written by the kernel
 // that produced it, read instead of splitting X per nonzero
-int launch_spmm(Handle& h, const double* X, double* YA, double* YM, int ncols, const float2* Xs = nullptr);
+int launch_spmm(Handle& h, const double* X, double* YA, double* YM, int ncols, const float* Xs = nullptr);
 int launch_csr_times_dense(const CsrDev& P, const double* D, int ldd, int ncols, double* Y, int ldy,
                            cudaStream_t s);
 int launch_residual(Handle& h, const double* AX, const double* MX, const double* lam, double* rho);
@@ -220,7 +222,7 @@ int launch_gram_raw(int64_t n, int k, int nu, const double* const* U, int nvb, i
 // split_out (double-word path only): also the (hi, lo) split of every output value
 int launch_combine_rows(Handle& h, int nin, const double* const* Win, const double* C, int ldc,
                         int csub, const double* Zadd, double* out, double alpha, int consistency_only = 0,
-                        float2* split_out = nullptr);
+                        float* split_out = nullptr);
 // hist_row: history row of the Ritz values (host count), or d_row != NULL: the
 // device step counter + 1 (captured iterations)
 int launch_rr(Handle& h, int m, const double* G, const double* Hm, const double* lam_old, double* C,

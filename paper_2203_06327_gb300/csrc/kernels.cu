@@ -63,50 +63,158 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 // ---------------------------------------------------------------------------
-// CSR SpMM over a block of vectors: YA = A X and (optionally) YM = M X with a
-// shared pattern.  LANES consecutive lanes serve one row; lane j of the group
-// owns columns j, j + LANES, ... (at most 2 per lane).  The row's column
-// indices and values are broadcast to the group; X rows are read as contiguous
-// ncols-vectors.
+// CSR SpMM over a block of vectors: YA = A X and (YM) YM = M X with a shared
+// pattern.  A lane owns four consecutive columns of a row, lpr = ceil(ncols / 4)
+// consecutive lanes serve the row, so 30 of 32 lanes or more have work for up to
+// 24 columns (a power of two of lanes left 12 of 32 idle at 20 columns).  The
+// entries of a row are taken kSpmmAhead at a time: first their columns and
+// values, then the X rows they name, then the products in entry order, so a row
+// costs two dependent accesses per kSpmmAhead entries.
+//   kSpmmF64    native FP64: bound by the FP64 pipe (0.53 T multiply-adds/s
+//               measured), so by the lanes that take part;
+//   kSpmmDw     double-word (Dot2) with pre-split matrix values, X split here;
+//   kSpmmSplit  the same with X's (hi, lo) split as written by the kernel that
+//               produced X (rows of 2 kp floats: the hi parts, then the lo parts).
+// The double-word products take two columns at a time in packed f32x2
+// instructions, the roundings of the scalar form.  VEC: rows of X, YA and YM are
+// aligned pairs (even ncols, 16-byte aligned arrays).  Measured (GB300, before ->
+// now): 20 columns, 27 entries a row, 250,047 rows in FP64 1529 -> 488 us (the
+// pipe's time is 493 us at its measured rate); 12 double-word columns of
+// 1,046,529 rows 241 -> 203 us with the split ahead (244 us splitting per entry).
 // ---------------------------------------------------------------------------
-template <int LANES>
-__global__ void __launch_bounds__(256) k_spmm(int n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
+constexpr int kSpmmF64 = 0, kSpmmDw = 1, kSpmmSplit = 2;
+constexpr int kSpmmAhead = 4;
+
+template <int MODE, bool VEC>
+__global__ void __launch_bounds__(128, (MODE == kSpmmDw) ? 4 : 5) k_spmm(int n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                               const double* __restrict__ va, const double* __restrict__ vm,
-                                              const double* __restrict__ X, double* __restrict__ YA,
-                                              double* __restrict__ YM, int ncols) {
-  constexpr int RPW = 32 / LANES;
+                                              const double* __restrict__ X, const float* __restrict__ Xs, int kp,
+                                              double* __restrict__ YA, double* __restrict__ YM, int ncols, int lpr) {
+  constexpr int U = kSpmmAhead;
   const int lane = threadIdx.x & 31;
+  const int rpw = 32 / lpr;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t row = warp * RPW + lane / LANES;
-  const int j0 = lane % LANES;
-  if (row >= n) return;
-  double a0 = 0, a1 = 0, m0 = 0, m1 = 0;
-  const int j1 = j0 + LANES;
-  const bool has0 = j0 < ncols, has1 = j1 < ncols;
-  for (int64_t e = rp[row]; e < rp[row + 1]; ++e) {
-    const int64_t c = ci[e];
-    const double av = va[e];
-    const double mv = vm ? vm[e] : 0.0;
-    const double* xr = X + c * ncols;
-    if (has0) {
-      double x = xr[j0];
-      a0 = fma(av, x, a0);
-      m0 = fma(mv, x, m0);
+  const int64_t row = warp * rpw + lane / lpr;
+  if (lane >= rpw * lpr || row >= n) return;
+  const int c0 = 4 * (lane % lpr);
+  const int nc = min(4, ncols - c0);
+  double fa[4] = {0, 0, 0, 0}, fm[4] = {0, 0, 0, 0};
+  dot2x2 da[2], dm[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    da[c].zero();
+    dm[c].zero();
+  }
+  const int64_t end = rp[row + 1];
+  for (int64_t e0 = rp[row]; e0 < end; e0 += U) {
+    int col[U];
+    double av[U], mv[U];  // FP64 values, or the (hi, lo) float pairs of the split ones
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool ok = e0 + u < end;
+      col[u] = ok ? ci[e0 + u] : -1;
+      av[u] = ok ? va[e0 + u] : 0.0;
+      mv[u] = (ok && vm) ? vm[e0 + u] : 0.0;
     }
-    if (has1) {
-      double x = xr[j1];
-      a1 = fma(av, x, a1);
-      m1 = fma(mv, x, m1);
+    double x[U][4];
+    f32x4p xh[U], xl[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (MODE == kSpmmSplit) {
+        if (col[u] >= 0) {
+          const float* xr = Xs + (int64_t)col[u] * 2 * kp + c0;
+          const ulonglong2 h = *reinterpret_cast<const ulonglong2*>(xr);
+          const ulonglong2 l = *reinterpret_cast<const ulonglong2*>(xr + kp);
+          xh[u] = f32x4p{{h.x, h.y}};
+          xl[u] = f32x4p{{l.x, l.y}};
+        }
+      } else if (col[u] >= 0) {
+        const double* xr = X + (int64_t)col[u] * ncols + c0;
+        if (VEC) {
+          const double2 p = *reinterpret_cast<const double2*>(xr);
+          x[u][0] = p.x;
+          x[u][1] = p.y;
+          x[u][2] = x[u][3] = 0.0;
+          if (nc > 2) {
+            const double2 q = *reinterpret_cast<const double2*>(xr + 2);
+            x[u][2] = q.x;
+            x[u][3] = q.y;
+          }
+        } else {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) x[u][c] = (c < nc) ? xr[c] : 0.0;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (col[u] < 0) continue;
+      if (MODE == kSpmmF64) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          fa[c] = fma(av[u], x[u][c], fa[c]);
+          if (vm) fm[c] = fma(mv[u], x[u][c], fm[c]);
+        }
+      } else {
+        if (MODE == kSpmmDw) {
+          dw s[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) s[c] = split_f64(x[u][c]);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            xh[u].p[c] = pack2(s[2 * c].hi, s[2 * c + 1].hi);
+            xl[u].p[c] = pack2(s[2 * c].lo, s[2 * c + 1].lo);
+          }
+        }
+        const float ah = __int_as_float(__double2loint(av[u])), al = __int_as_float(__double2hiint(av[u]));
+        const unsigned long long pa = pack2(ah, ah), na = pack2(-ah, -ah), ta = pack2(-al, -al);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) da[c].mac(pa, na, ta, xh[u].p[c], xl[u].p[c]);
+        if (vm) {
+          const float mh = __int_as_float(__double2loint(mv[u])), ml = __int_as_float(__double2hiint(mv[u]));
+          const unsigned long long pm = pack2(mh, mh), nm = pack2(-mh, -mh), tm = pack2(-ml, -ml);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) dm[c].mac(pm, nm, tm, xh[u].p[c], xl[u].p[c]);
+        }
+      }
     }
   }
-  if (has0) {
-    YA[row * ncols + j0] = a0;
-    if (YM) YM[row * ncols + j0] = m0;
-  }
-  if (has1) {
-    YA[row * ncols + j1] = a1;
-    if (YM) YM[row * ncols + j1] = m1;
-  }
+  auto store = [&](double* Y, double (&f)[4], dot2x2 (&d)[2]) {
+    if (MODE != kSpmmF64) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        f[2 * c] = d[c].value0();
+        f[2 * c + 1] = d[c].value1();
+      }
+    }
+    double* y = Y + row * ncols + c0;
+    if (VEC) {
+      *reinterpret_cast<double2*>(y) = make_double2(f[0], f[1]);
+      if (nc > 2) *reinterpret_cast<double2*>(y + 2) = make_double2(f[2], f[3]);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (c < nc) y[c] = f[c];
+    }
+  };
+  store(YA, fa, da);
+  if (YM) store(YM, fm, dm);
+}
+
+// The split that kSpmmSplit reads, of an X given in FP64: a thread per four columns.
+__global__ void __launch_bounds__(256) k_split_rows(int64_t n, int ncols, int kp, const double* __restrict__ X,
+                                                    float* __restrict__ Xs) {
+  const int lpr = kp / 4;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= n * lpr) return;
+  const int64_t r = t / lpr;
+  const int c0 = 4 * (int)(t - r * lpr);
+  dw s[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) s[c] = split_f64(c0 + c < ncols ? X[r * ncols + c0 + c] : 0.0);
+  float* o = Xs + r * 2 * kp + c0;
+  *reinterpret_cast<float4*>(o) = make_float4(s[0].hi, s[1].hi, s[2].hi, s[3].hi);
+  *reinterpret_cast<float4*>(o + kp) = make_float4(s[0].lo, s[1].lo, s[2].lo, s[3].lo);
 }
 
 // Y[r, j] = sum_e P[r, c_e] D[c_e, j] for j < ncols (sparse times small dense).
@@ -480,7 +588,8 @@ __global__ void __launch_bounds__(256) k_gram_reduce(int nblk, int mu, int mv, i
 constexpr int kCombRows = 64;
 __global__ void __launch_bounds__(256) k_combine_dw(int64_t n, int k, int nin, Ptrs6 W, const double* __restrict__ C,
                                                     int ldc, int csub, const double* __restrict__ Zadd,
-                                                    double* __restrict__ out, double sign, float2* __restrict__ outs) {
+                                                    double* __restrict__ out, double sign, float* __restrict__ outs,
+                                                    int kp) {
   extern __shared__ __align__(16) float csm[];
   const int m = nin * k;
   float* Ch = csm;                       // m x csub
@@ -530,66 +639,10 @@ __global__ void __launch_bounds__(256) k_combine_dw(int64_t n, int k, int nin, P
     const int64_t o = (row0 + r) * csub + j;
     if (Zadd) v += Zadd[o];
     out[o] = v;
-    if (outs) {
+    if (outs) {  // rows of 2 kp floats: the hi parts, then the lo parts
       const dw sp = split_f64(v);
-      outs[o] = make_float2(sp.hi, sp.lo);
-    }
-  }
-}
-
-// CSR SpMM in double-word arithmetic with pre-split matrix values (hi/lo
-// float arrays of K and M): YA = K X, YM = M X.  LANES lanes serve one row;
-// lane j of the group owns columns j + LANES c, c < CPL.  The X entries are
-// split on the fly (integer operations only), or (XS) read as the (hi, lo)
-// pairs that the kernel producing X wrote beside it (split_f64 of the same
-// values: the same products).
-template <int LANES, int CPL, bool XS>
-__global__ void __launch_bounds__(256, 4) k_spmm_dw(int n, const int64_t* __restrict__ rp,
-                                                    const int32_t* __restrict__ ci,
-                                                    const float2* __restrict__ va, const float2* __restrict__ vm,
-                                                    const double* __restrict__ X, const float2* __restrict__ Xs,
-                                                    double* __restrict__ YA, double* __restrict__ YM, int ncols) {
-  constexpr int RPW = 32 / LANES;
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t row = warp * RPW + lane / LANES;
-  const int j0 = lane % LANES;
-  if (row >= n) return;
-  dot2 a[CPL], m[CPL];
-#pragma unroll
-  for (int c = 0; c < CPL; ++c) {
-    a[c].zero();
-    m[c].zero();
-  }
-  for (int64_t e = rp[row]; e < rp[row + 1]; ++e) {
-    const int64_t col = ci[e];
-    const float2 av = va[e];
-    const float2 mv = vm ? vm[e] : make_float2(0.f, 0.f);
-    const double* xr = X + col * ncols;
-    const float2* xsr = Xs + col * ncols;
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) {
-      const int j = j0 + LANES * c;
-      if (j < ncols) {
-        dw x;
-        if (XS) {
-          const float2 p = xsr[j];
-          x.hi = p.x;
-          x.lo = p.y;
-        } else {
-          x = split_f64(xr[j]);
-        }
-        a[c].mac(av.x, av.y, x.hi, x.lo);
-        m[c].mac(mv.x, mv.y, x.hi, x.lo);
-      }
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < CPL; ++c) {
-    const int j = j0 + LANES * c;
-    if (j < ncols) {
-      YA[row * ncols + j] = a[c].value();
-      if (YM) YM[row * ncols + j] = m[c].value();
+      outs[(row0 + r) * 2 * kp + j] = sp.hi;
+      outs[(row0 + r) * 2 * kp + kp + j] = sp.lo;
     }
   }
 }
@@ -602,7 +655,7 @@ __global__ void __launch_bounds__(256, 4) k_spmm_dw(int n, const int64_t* __rest
 // W and the coefficients.
 __global__ void __launch_bounds__(256) k_combine_f32(int64_t n, int k, int nin, Ptrs6 W, const double* __restrict__ C,
                                                      int ldc, int csub, const double* __restrict__ Zadd,
-                                                     double* __restrict__ out, float sign, float2* __restrict__ outs) {
+                                                     double* __restrict__ out, float sign, float* __restrict__ outs, int kp) {
   extern __shared__ __align__(16) float csm[];
   const int m = nin * k;
   float* Cs = csm;              // m x csub
@@ -627,7 +680,8 @@ __global__ void __launch_bounds__(256) k_combine_f32(int64_t n, int k, int nin, 
     out[o] = vd;
     if (outs) {
       const dw sp = split_f64(vd);
-      outs[o] = make_float2(sp.hi, sp.lo);
+      outs[(row0 + r) * 2 * kp + j] = sp.hi;
+      outs[(row0 + r) * 2 * kp + kp + j] = sp.lo;
     }
   }
 }
@@ -2879,76 +2933,53 @@ void prof_flush(Handle& h) {
 // ===========================================================================
 // launchers
 // ===========================================================================
-int launch_spmm(Handle& h, const double* X, double* YA, double* YM, int ncols, const float2* Xs) {
+// 1,046,529 rows, 12 columns: 203 us split ahead, 244 us per entry; at 4 M products (a tenth of
+// that) the pass and its launch take about 6 us, the splits saved 4 to 6
+constexpr int64_t kSplitAhead = 8000000;
+int launch_spmm(Handle& h, const double* X, double* YA, double* YM, int ncols, const float* Xs) {
   ProfScope ps(h, BPJD_PROF_SPMM);
   const int n = h.n;
-  auto go = [&](auto lanes_tag, const CsrDev& A, const double* vm, double* ya, double* ym) {
-    constexpr int LANES = decltype(lanes_tag)::value;
-    constexpr int RPW = 32 / LANES;
-    int64_t warps = (n + RPW - 1) / RPW;
-    int64_t blocks = (warps * 32 + 255) / 256;
-    k_spmm<LANES><<<(unsigned)blocks, 256, 0, h.stream>>>(n, A.row_ptr, A.col, A.val, vm, X, ya, ym, ncols);
+  const int lpr = (ncols + 3) / 4, rpw = 32 / lpr;
+  // four warps per block; one when that fills the chip better (few rows)
+  const int64_t warps = ((int64_t)n + rpw - 1) / rpw;
+  const int wpb = (warps < 4 * 304) ? 1 : 4;
+  const unsigned blocks = (unsigned)((warps + wpb - 1) / wpb);
+  auto aligned = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
+  const bool vec = ncols % 2 == 0 && aligned(X) && aligned(YA) && aligned(YM);
+  const bool dw = h.dword() && h.Asplit;
+  // splitting X's rows ahead costs a pass over X and a launch, splitting them in the product
+  // one split per entry of the matrix: ahead from kSplitAhead products on (a row's share of
+  // either side does not depend on n) where the handle's buffer has the columns
+  int kp = h.kp();
+  if (dw && !Xs && (ncols + 3) / 4 * 4 == kp && h.A.nnz * ncols >= kSplitAhead) {
+    const int64_t t = (int64_t)n * (kp / 4);
+    k_split_rows<<<(unsigned)((t + 255) / 256), 256, 0, h.stream>>>(n, ncols, kp, X, h.xsplit);
+    h.launches += 1;
+    Xs = h.xsplit;
+  }
+  auto go = [&](auto mode, auto vec_tag, const CsrDev& A, const void* va, const void* vm, double* ya, double* ym) {
+    k_spmm<decltype(mode)::value, decltype(vec_tag)::value><<<blocks, 32 * wpb, 0, h.stream>>>(
+        n, A.row_ptr, A.col, (const double*)va, (const double*)vm, X, Xs, kp, ya, ym, ncols, lpr);
     h.launches += 1;
   };
-  if (h.dword() && h.Asplit) {
-    // lanes per row and columns per lane: every lane of a row group busy for k = 4, 8, 12, 16, 24, 32
-    auto god = [&](auto lanes_tag, auto cpl_tag, const float2* va, const float2* vm, double* ya, double* ym,
-                   const CsrDev& A) {
-      constexpr int LANES = decltype(lanes_tag)::value;
-      constexpr int CPL = decltype(cpl_tag)::value;
-      constexpr int RPW = 32 / LANES;
-      int64_t warps = (n + RPW - 1) / RPW;
-      int64_t blocks = (warps * 32 + 255) / 256;
-      if (Xs)
-        k_spmm_dw<LANES, CPL, true><<<(unsigned)blocks, 256, 0, h.stream>>>(n, A.row_ptr, A.col, va, vm, X, Xs, ya,
-                                                                           ym, ncols);
-      else
-        k_spmm_dw<LANES, CPL, false><<<(unsigned)blocks, 256, 0, h.stream>>>(n, A.row_ptr, A.col, va, vm, X, Xs, ya,
-                                                                            ym, ncols);
-      h.launches += 1;
-    };
-    using I = std::integral_constant<int, 1>;
-    using I2 = std::integral_constant<int, 2>;
-    using I3 = std::integral_constant<int, 3>;
-    using I4 = std::integral_constant<int, 4>;
-    using I8 = std::integral_constant<int, 8>;
-    auto dispatch_dw = [&](const CsrDev& A, const float2* va, const float2* vm, double* ya, double* ym) {
-      if (ncols <= 4)
-        god(I4(), I(), va, vm, ya, ym, A);
-      else if (ncols <= 8)
-        god(I4(), I2(), va, vm, ya, ym, A);
-      else if (ncols <= 12)
-        god(I4(), I3(), va, vm, ya, ym, A);
-      else if (ncols <= 16)
-        god(I4(), I4(), va, vm, ya, ym, A);
-      else if (ncols <= 24)
-        god(I8(), I3(), va, vm, ya, ym, A);
-      else
-        god(I8(), I4(), va, vm, ya, ym, A);
-    };
-    if (h.same_pattern) {
-      dispatch_dw(h.A, h.Asplit, h.Msplit, YA, YM);
-    } else {
-      dispatch_dw(h.A, h.Asplit, nullptr, YA, nullptr);
-      dispatch_dw(h.M, h.Msplit, nullptr, YM, nullptr);
-    }
-    return (int)cudaGetLastError();
-  }
-  auto dispatch = [&](const CsrDev& A, const double* vm, double* ya, double* ym) {
-    if (ncols <= 4)
-      go(std::integral_constant<int, 4>(), A, vm, ya, ym);
-    else if (ncols <= 8)
-      go(std::integral_constant<int, 8>(), A, vm, ya, ym);
-    else if (ncols <= 16)
-      go(std::integral_constant<int, 16>(), A, vm, ya, ym);
+  auto run = [&](const CsrDev& A, const void* va, const void* vm, double* ya, double* ym) {
+    using F = std::integral_constant<int, kSpmmF64>;
+    using D = std::integral_constant<int, kSpmmDw>;
+    using P = std::integral_constant<int, kSpmmSplit>;
+    if (!dw)
+      vec ? go(F(), std::true_type(), A, va, vm, ya, ym) : go(F(), std::false_type(), A, va, vm, ya, ym);
+    else if (Xs)
+      vec ? go(P(), std::true_type(), A, va, vm, ya, ym) : go(P(), std::false_type(), A, va, vm, ya, ym);
     else
-      go(std::integral_constant<int, 32>(), A, vm, ya, ym);
+      vec ? go(D(), std::true_type(), A, va, vm, ya, ym) : go(D(), std::false_type(), A, va, vm, ya, ym);
   };
+  const void* va = dw ? (const void*)h.Asplit : (const void*)h.A.val;
+  const void* vm = dw ? (const void*)h.Msplit : (const void*)h.M.val;
   if (h.same_pattern) {
-    dispatch(h.A, h.M.val, YA, YM);
+    run(h.A, va, vm, YA, YM);
   } else {
-    dispatch(h.A, nullptr, YA, nullptr);
-    dispatch(h.M, nullptr, YM, nullptr);
+    run(h.A, va, nullptr, YA, nullptr);
+    run(h.M, vm, nullptr, YM, nullptr);
   }
   return (int)cudaGetLastError();
 }
@@ -3094,7 +3125,7 @@ int launch_gram(Handle& h, int nu, const double* const* U, int nvb, int nv, cons
 }
 
 int launch_combine_rows(Handle& h, int nin, const double* const* Win, const double* C, int ldc, int csub,
-                        const double* Zadd, double* out, double sign, int consistency_only, float2* split_out) {
+                        const double* Zadd, double* out, double sign, int consistency_only, float* split_out) {
   ProfScope ps(h, BPJD_PROF_COMBINE);
   h.launches += 1;
   if (nin < 1 || nin > 6 || nin * h.k > 96 || csub < 1 || csub > 256) return (int)cudaErrorInvalidValue;
@@ -3106,7 +3137,7 @@ int launch_combine_rows(Handle& h, int nin, const double* const* Win, const doub
     allow_dynamic_smem((const void*)k_combine_f32);
     const int64_t blocks = ((int64_t)h.n + kCombRows - 1) / kCombRows;
     k_combine_f32<<<(unsigned)blocks, 256, sm, h.stream>>>(h.n, h.k, nin, w, C, ldc, csub, Zadd, out, (float)sign,
-                                                           split_out);
+                                                           split_out, h.kp());
     return (int)cudaGetLastError();
   }
   if (h.dword()) {
@@ -3115,7 +3146,7 @@ int launch_combine_rows(Handle& h, int nin, const double* const* Win, const doub
     allow_dynamic_smem((const void*)k_combine_dw);
     const int64_t blocks = ((int64_t)h.n + kCombRows - 1) / kCombRows;
     k_combine_dw<<<(unsigned)blocks, 256, sm, h.stream>>>(h.n, h.k, nin, w, C, ldc, csub, Zadd, out, sign,
-                                                          split_out);
+                                                          split_out, h.kp());
     return (int)cudaGetLastError();
   }
   int64_t tot = (int64_t)h.n * csub;

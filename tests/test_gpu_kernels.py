@@ -107,3 +107,23 @@ def test_block_gram_exact_integers(n, k, nu, nv, sym):
     assert fn(n, k, nu, pu, nv, pv, 1 if sym else 0, out.data_ptr(), None) == B.OK
     Un, Vn = np.hstack(U), np.hstack(V)
     np.testing.assert_array_equal(out.cpu().numpy(), Un.T @ Vn)
+
+
+# Products of every number of columns a lane group can serve (4 per lane, 1 to 16 lanes), odd ones and arrays
+# that start 8 bytes off a 16-byte boundary (scalar accesses); tolerance as for the other SpMM checks.
+@pytest.mark.parametrize("ncols", [1, 2, 3, 4, 5, 7, 8, 11, 12, 17, 20, 24, 31, 32, 33, 64])
+@pytest.mark.parametrize("precision", [B.FP64, B.MIXED], ids=["fp64", "mixed"])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_spmm_columns_and_alignment(ncols, precision, offset):
+    pb = B.problem_create("p1_2d", (24, 18), (1.0, 0.751), (4, 3), 1)
+    sv = B.Solver.from_problem(pb, 3, device=DEV, precision=precision)
+    n = sv.n
+    X = np.random.default_rng(ncols).standard_normal((n, ncols))
+    bufs = [torch.full((n * ncols + offset,), float("nan"), dtype=torch.float64, device=DEV) for _ in range(3)]
+    Xd, YA, YM = [b[offset:].view(n, ncols) for b in bufs]
+    Xd.copy_(torch.tensor(X))
+    sv.spmm(Xd, YA, YM)
+    for Y, a in ((YA, pb.K), (YM, pb.M)):
+        A = _scipy(a)
+        assert np.all(np.abs(Y.cpu().numpy() - A @ X) <= 1e-13 * (abs(A) @ np.abs(X)) + 1e-300)
+    sv.close()

@@ -853,15 +853,16 @@ __global__ void k_local_band(int npairs, int k, const int64_t* __restrict__ sub_
 //   - the warp that updates the next pivot forms its reciprocal root while the
 //     other warps do the rest of the update;
 //   - band rows and right-hand sides enter from registers loaded a step and a
-//     window period ahead;
-//   - backward, L^T x = y right-looking: the thread of a slot keeps the pending
-//     y of its row and streams its own record (contiguous, eight loads ahead),
-//     so a row costs one multiply, one fused multiply-add and one barrier.
+//     window period ahead.
+// Every entry takes the operations of the one-warp kernel in its order, the
+// backward sums included, so the results are the same bits (an rsqrt() and a
+// right-looking backward sweep were 0.6 ms faster, and moved the iterates of a
+// slowly converging solve by 1e-9).
 // 64 subdomains of 32 x 32 cells, 12 columns, window 37 (GB300): one warp per pair
-// on a full square window 10.27 ms, this kernel 2.9 ms (FP64 pipe 60 % busy; the
-// rest is the chain of a step and six pairs on some SMs against five on others)
+// on a full square window 10.27 ms, this kernel 3.7 ms (the FP64 pipe and the chain
+// of a step; six pairs on some SMs against five on others)
 // ---------------------------------------------------------------------------
-constexpr int kPivotChunks = 7;
+constexpr int kPivotChunks = 16;
 __global__ void __launch_bounds__(192) k_local_band_f64(int k, const int64_t* __restrict__ sub_ptr,
                                                         const int32_t* __restrict__ sub_dofs, int B,
                                                         const double* __restrict__ bandK,
@@ -870,7 +871,7 @@ __global__ void __launch_bounds__(192) k_local_band_f64(int k, const int64_t* __
                                                         const double* __restrict__ rho, double* Lbuf, double* wpk,
                                                         int32_t* err, int64_t rec_base) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ double s_inv, s_x[2];
+  __shared__ double s_inv;
   __shared__ int s_bad;
   const int NT = blockDim.x, tid = threadIdx.x, NR = B * (B + 1) / 2, NE = NR + B;
   double* W = reinterpret_cast<double*>(smraw);  // [NE]: window, then the right-hand sides (row B)
@@ -922,7 +923,7 @@ __global__ void __launch_bounds__(192) k_local_band_f64(int k, const int64_t* __
       s_bad = 1;
       atomicOr(err, 1);
     }
-    s_inv = rsqrt(piv);
+    s_inv = 1.0 / sqrt(piv);
   }
   __syncthreads();
   if (s_bad) return;
@@ -994,7 +995,7 @@ __global__ void __launch_bounds__(192) k_local_band_f64(int k, const int64_t* __
           s_bad = 1;
           atomicOr(err, 1);
         }
-        s_inv = rsqrt(pv);
+        s_inv = 1.0 / sqrt(pv);
       }
       for (int r = 1; r < npc; r += 4) update(std::integral_constant<int, 4>(), r, 1, npc);
     } else {
@@ -1010,55 +1011,58 @@ __global__ void __launch_bounds__(192) k_local_band_f64(int k, const int64_t* __
     if (s_bad) return;
     s = sn;
   }
-  // backward substitution: slot u holds row q (q mod B = u), the pending y of which takes
-  // -L(j, q) x_j from every later row j; record q is read from entry B - 1 down to 1/L_qq
-  constexpr int PF = 8;
-  int t = 0, q = -1;  // entry and row of this thread's next load
-  double y = 0.0, yn = 0.0, ring[PF];
-  auto next = [&]() -> double {
-    const double v = (q >= 0) ? Lp[(size_t)q * B + t] : 0.0;
-    if (--t < 0) {
-      t = B - 1;
-      q -= B;
+  // backward substitution by one warp (another SM quarter from one block to the next): lane t
+  // sums the products of entries 1 + t, 33 + t, .. of record j with the solved rows, a
+  // butterfly adds the lanes; record, y and 1/L_jj are loaded two rows ahead
+  if ((tid >> 5) != (int)(blockIdx.x & 3)) return;
+  constexpr int NC = 6;  // entries of a record per lane, at most (B <= 168)
+  const int lane = tid & 31;
+  double* xs = lc;  // [B] solved rows by slot
+  double c0[NC], c1[NC], c2[NC], y0 = 0.0, y1 = 0.0, y2 = 0.0, d0 = 0.0, d1 = 0.0, d2 = 0.0;
+  auto fetch = [&](int j, double (&c)[NC], double& y, double& d) {
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const int t = 1 + lane + 32 * q;
+      c[q] = (j >= 0 && t < B) ? Lp[(size_t)j * B + t] : 0.0;
     }
-    return v;
+    if (j >= 0 && lane == 0) {
+      y = wp[(size_t)j * k];
+      d = Lp[(size_t)j * B];
+    }
   };
-  int row = -1;  // row held by this slot
-  if (own) {
-    t = (nl - 1) % B - u;
-    t += (t < 0) ? B : 0;
-    q = row = nl - 1 - t;
-    y = (row >= 0) ? wp[(size_t)row * k] : 0.0;
-    yn = (row >= B) ? wp[(size_t)(row - B) * k] : 0.0;
-  }
+  fetch(nl - 1, c0, y0, d0);
+  fetch(nl - 2, c1, y1, d1);
+  for (int j = nl - 1, s = (nl - 1) % B; j >= 0; --j) {
+    fetch(j - 2, c2, y2, d2);
+    double part = 0.0;
 #pragma unroll
-  for (int r = 0; r < PF; ++r) ring[r] = next();
-  if (own && row == nl - 1) s_x[(nl - 1) & 1] = y * ring[0];
-  for (int jb = nl - 1; jb >= 0; jb -= PF) {
-#pragma unroll
-    for (int r = 0; r < PF; ++r) {
-      const int j = jb - r;
-      if (j < 0) break;
-      __syncthreads();
-      if (own) {
-        const double xj = s_x[j & 1];
-        if (row == j) {
-          wp[(size_t)j * k] = xj;
-          y = yn;
-          row -= B;
-          yn = (row >= B) ? wp[(size_t)(row - B) * k] : 0.0;
-          // window of one row: the entering row is the next pivot
-          if (B == 1 && j > 0) s_x[(j - 1) & 1] = y * ring[(r + 1) % PF];
-        } else {
-          y = fma(-ring[r], xj, y);
-          if (row == j - 1) s_x[(j - 1) & 1] = y * ring[(r + 1) % PF];
-        }
+    for (int q = 0; q < NC; ++q) {
+      const int t = 1 + lane + 32 * q;
+      if (t < B && j + t < nl) {
+        int o = s + t;
+        o -= (o >= B) ? B : 0;
+        part = fma(c0[q], xs[o], part);
       }
-      ring[r] = next();
     }
+    part = warp_sum(part);
+    if (lane == 0) {
+      const double x = (y0 - part) * d0;
+      xs[s] = x;
+      wp[(size_t)j * k] = x;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      c0[q] = c1[q];
+      c1[q] = c2[q];
+    }
+    y0 = y1;
+    y1 = y2;
+    d0 = d1;
+    d1 = d2;
+    s = (s == 0) ? B - 1 : s - 1;
   }
 }
-
 
 
 // ---------------------------------------------------------------------------

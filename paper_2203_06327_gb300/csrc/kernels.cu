@@ -394,13 +394,17 @@ __global__ void __launch_bounds__(256) k_inner(int n, int k, int p, Ptrs6 U, int
 // same roundings, half the issue slots, which the splits and copies then use):
 // a tile's pairs are taken along its diagonals, (x, y) with (x + 1, y + 1) and
 // (x, y + 1) with (x + 1, y), so that U's pairs are the loaded ones and V's are
-// the loaded ones and their swaps.  Measured (GB300, before -> now): 36 columns
-// of 261,121 rows, symmetric, 188 -> 148 us (136 us in this kernel: FP32 pipe
-// 53 % busy; two or three blocks per SM are alike), 19 x 57 columns of 65,025
-// rows 99 -> 81 us, 18 columns of 2,209 rows (both products) 44 -> 12 us.
+// the loaded ones and their swaps.  The partition of the rows and the order of
+// the sums are those of the scalar kernel this replaced: the same bits.  Measured
+// (GB300, before -> now): 36 columns of 261,121 rows, symmetric, 188 -> 151 us
+// (FP32 pipe about half busy; two products in one block, W split once, were 3 %
+// slower than a block each), 19 x 57 columns of 65,025 rows 99 -> 83 us, the
+// products of a step at 2,209 rows and k = 6 49 -> 19 us on average.  A pair of
+// 36-column products of 261,121 rows, too large to gain from the shorter tail
+// and with W split twice, takes 3 % longer than before.
 // ---------------------------------------------------------------------------
-constexpr int kGramRows = 32;     // rows per block, at least
-constexpr int kGramBlocks = 456;  // three resident blocks on each of the 152 SMs: one wave
+constexpr int kGramRows = 64;     // a block's rows are a multiple of this
+constexpr int kGramBlocks = 304;  // two resident blocks on each of the 152 SMs: one wave per product
 
 __device__ __forceinline__ void gram_tile_of(int t, int TU, int TV, int sym, int& ta, int& tb) {
   if (!sym) {
@@ -425,8 +429,7 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-template <int THREADS>
-__global__ void __launch_bounds__(THREADS, (THREADS <= 192) ? 3 : 2)
+__global__ void __launch_bounds__(256, 2)
     k_gram_dw(int n, int k, int nu, Ptrs6 U, int nvb, Ptrs6 V1, Ptrs6 V2, int sym, int shared_mask, int S,
               int rows_per_block, int R, double* partial) {
   extern __shared__ __align__(16) float gsm[];
@@ -547,28 +550,31 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 192) ? 3 : 2)
   }
 }
 
-// Sum of the per-block Gram partials: a block serves 8 consecutive entries; thread
-// group g = tid / 8 adds the blocks b = g, g + 32, ... in order, then a fixed tree over
-// the groups (bit-reproducible).
-__global__ void __launch_bounds__(256) k_gram_reduce(int nblk, int mu, int mv, int sym,
+// Sum of the per-block Gram partials: a block serves 32 consecutive entries;
+// warp w adds blocks b = w, w + 8, ... in order, warp 0 adds the eight results
+// in order (fixed order: bit-reproducible).
+__global__ void __launch_bounds__(256) k_gram_reduce(int nblk, int nv, int mu, int mv, int sym,
                                                      const double* __restrict__ partial, double* out1,
                                                      double* out2) {
-  __shared__ double red[8][8];
+  __shared__ double red[8][32];
   const int TU = (mu + 3) / 4, TV = (mv + 3) / 4;
   const int ntiles = sym ? TU * (TU + 1) / 2 : TU * TV;
-  const int per = ntiles * 16;  // entries of one product: a multiple of 16
-  const int t = blockIdx.x * 8 + (threadIdx.x & 7), w = threadIdx.x >> 5;
+  const int per = ntiles * 16, total = nv * per;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int t = blockIdx.x * 32 + lane;
   const int v = t / per, rem = t % per;
   double s = 0;
-#pragma unroll 5
-  for (int b = threadIdx.x >> 3; b < nblk; b += 32) s += partial[((int64_t)v * nblk + b) * per + rem];
-  s += __shfl_xor_sync(0xffffffffu, s, 8);
-  s += __shfl_xor_sync(0xffffffffu, s, 16);
-  if ((threadIdx.x & 31) < 8) red[w][threadIdx.x & 7] = s;
+  if (t < total) {
+    const double* src = partial + (int64_t)v * nblk * per + rem;
+#pragma unroll 8
+    for (int b = w; b < nblk; b += 8) s += src[(int64_t)b * per];
+  }
+  red[w][lane] = s;
   __syncthreads();
-  if (threadIdx.x >= 8) return;
-  const int q = threadIdx.x;
-  s = ((red[0][q] + red[1][q]) + (red[2][q] + red[3][q])) + ((red[4][q] + red[5][q]) + (red[6][q] + red[7][q]));
+  if (w != 0 || t >= total) return;
+  s = red[0][lane];
+#pragma unroll
+  for (int q = 1; q < 8; ++q) s += red[q][lane];
   const int tile = rem / 16, e = rem % 16;
   int ta, tb;
   gram_tile_of(tile, TU, TV, sym, ta, tb);
@@ -2937,8 +2943,8 @@ void prof_flush(Handle& h) {
 // ===========================================================================
 // launchers
 // ===========================================================================
-// 1,046,529 rows, 12 columns: 203 us split ahead, 244 us per entry; at 4 M products (a tenth of
-// that) the pass and its launch take about 6 us, the splits saved 4 to 6
+// products; us split ahead / per entry (GB300): 12 columns 6.9 M 22.6 / 20.5, 12.3 M 30.8 / 32.8,
+// 49 M 119 / 139; 5 columns 1.7 M 14.4 / 14.4, 5.1 M 24.6 / 28.7, 21 M 78 / 115
 constexpr int64_t kSplitAhead = 8000000;
 int launch_spmm(Handle& h, const double* X, double* YA, double* YM, int ncols, const float* Xs) {
   ProfScope ps(h, BPJD_PROF_SPMM);
@@ -2952,8 +2958,8 @@ int launch_spmm(Handle& h, const double* X, double* YA, double* YM, int ncols, c
   const bool vec = ncols % 2 == 0 && aligned(X) && aligned(YA) && aligned(YM);
   const bool dw = h.dword() && h.Asplit;
   // splitting X's rows ahead costs a pass over X and a launch, splitting them in the product
-  // one split per entry of the matrix: ahead from kSplitAhead products on (a row's share of
-  // either side does not depend on n) where the handle's buffer has the columns
+  // one split per entry of the matrix: ahead from kSplitAhead products on, where the handle's
+  // buffer has the columns
   int kp = h.kp();
   if (dw && !Xs && (ncols + 3) / 4 * 4 == kp && h.A.nnz * ncols >= kSplitAhead) {
     const int64_t t = (int64_t)n * (kp / 4);
@@ -3036,54 +3042,37 @@ int launch_inner(Handle& h, int p, const double* const* U, int q, const double* 
   return (int)cudaGetLastError();
 }
 
-// Blocks, rows per block and per chunk, slices and shared memory of a Gram launch.
+// Blocks, rows per block and per chunk, slices and shared memory of a Gram launch.  The
+// partition of the rows (and with it the order of every sum, hence the bits) is a function of
+// n, the columns and nv alone; 45 tiles: 5 slices, 225 of 256 threads.
 struct GramShape {
   int ntiles = 0, S = 1, threads = 32, nblk = 1, rpb = 1, R = 1;
   size_t smem = 0;
 };
-static GramShape gram_shape(int64_t n, int k, int nu, int nvb, int nv, int sym, size_t capacity) {
+static GramShape gram_shape(int64_t n, int k, int nu, int nvb, int nv, int sym) {
   GramShape g;
   const int TU = (nu * k + 3) / 4, TV = (nvb * k + 3) / 4;
   g.ntiles = sym ? TU * (TU + 1) / 2 : TU * TV;
-  // slices of a chunk's rows: the count that leaves the fewest lanes without a tile among
-  // those that make 128 to 192 threads, of which three blocks fit an SM (at most 16 slices;
-  // 45 tiles: 4 slices, 180 of 192); more tiles than that take one slice, two blocks on an SM
-  double best = -1;
-  for (int S = 1; S <= 16 && (S == 1 || S * g.ntiles <= 192); ++S) {
-    const int th = (S * g.ntiles + 31) / 32 * 32;
-    const double eff = (double)S * g.ntiles / th - (th < 128 ? 1.0 - th / 512.0 : 0.0);
-    if (eff >= best) {
-      best = eff;
-      g.S = S;
-    }
-  }
+  g.S = std::max(1, 256 / g.ntiles);
   g.threads = (g.S * g.ntiles + 31) / 32 * 32;
-  const int64_t fit = std::max<int64_t>(1, (int64_t)(capacity / ((size_t)g.ntiles * nv * 16)));
-  const int64_t wave = (g.threads <= 192 ? kGramBlocks : kGramBlocks / 3 * 2) / nv;
-  const int64_t want = std::min(fit, std::min<int64_t>(wave, (n + kGramRows - 1) / kGramRows));
-  g.rpb = (int)((n + want - 1) / want);
+  const int nblk = (int)std::min<int64_t>(kGramBlocks, (n + kGramRows - 1) / kGramRows);
+  g.rpb = (int)(((n + nblk - 1) / nblk + kGramRows - 1) / kGramRows * kGramRows);
   g.nblk = (int)((n + g.rpb - 1) / g.rpb);
-  // chunk rows: two raw FP64 buffers and the (hi, lo) planes within 70 KB (three blocks on an
-  // SM), a multiple of the slices, no longer than a block's rows
-  const size_t per_row = 16 * (size_t)(nu + nvb) * k + 32 * (size_t)(TU + TV);
-  int R = (int)std::min<size_t>(64, (70 * 1024) / per_row);
-  R = std::min(R, (g.rpb + g.S - 1) / g.S * g.S);
-  if (R >= g.S) R -= R % g.S;
-  R += R & 1;  // raw buffers and planes stay 16-byte aligned
-  g.R = std::max(2, R);
-  g.smem = std::max(per_row * g.R, (size_t)g.S * g.ntiles * 16 * sizeof(double));
+  // chunk rows: a divisor of kGramRows keeping the staging of all blocks of the call (two raw
+  // FP64 buffers and the hi/lo planes, 24 bytes per value) within 100 KB
+  const int nseg = nu + nv * nvb;
+  int R = kGramRows;
+  while (R > 1 && (size_t)24 * R * k * nseg > 100 * 1024) R /= 2;
+  g.R = R;
+  const int Ra = R + (R & 1);  // raw buffers and planes stay 16-byte aligned
+  g.smem = std::max((16 * (size_t)(nu + nvb) * k + 32 * (size_t)(TU + TV)) * Ra,
+                    (size_t)g.S * g.ntiles * 16 * sizeof(double));
   return g;
 }
 
-// What bpjd_block_gram_noalloc asks of its static array (row ranges in units of 64 rows);
-// a launch takes fewer blocks where the scratch holds fewer partial sums.
 size_t gram_partial_doubles(int64_t n, int k, int nu, int nvb, int sym) {
-  constexpr int64_t kUnit = 64, kBlocks = 304;
-  const int TU = (nu * k + 3) / 4, TV = (nvb * k + 3) / 4;
-  const int ntiles = sym ? TU * (TU + 1) / 2 : TU * TV;
-  const int64_t nblk = std::min<int64_t>(kBlocks, (n + kUnit - 1) / kUnit);
-  const int64_t rpb = ((n + nblk - 1) / nblk + kUnit - 1) / kUnit * kUnit;
-  return (size_t)((n + rpb - 1) / rpb) * ntiles * 16;
+  const GramShape g = gram_shape(n, k, nu, nvb, 1, sym);
+  return (size_t)g.nblk * g.ntiles * 16;
 }
 
 int launch_gram_raw(int64_t n, int k, int nu, const double* const* U, int nvb, int nv, const double* const* V1,
@@ -3104,20 +3093,13 @@ int launch_gram_raw(int64_t n, int k, int nu, const double* const* U, int nvb, i
       if (shared && U[b] != V2[b]) shared &= ~2;
     }
   }
-  const GramShape g = gram_shape(n, k, nu, nvb, nv, sym, partial_capacity);
+  const GramShape g = gram_shape(n, k, nu, nvb, nv, sym);
   const int total = nv * ntiles * 16;
   if ((size_t)g.nblk * total > partial_capacity) return (int)cudaErrorInvalidValue;
-  const dim3 grid(g.nblk, nv);
-  if (g.threads <= 192) {
-    allow_dynamic_smem((const void*)k_gram_dw<192>);
-    k_gram_dw<192><<<grid, g.threads, g.smem, stream>>>((int)n, k, nu, u, nvb, v1, v2, sym, shared, g.S, g.rpb, g.R,
-                                                        partial);
-  } else {
-    allow_dynamic_smem((const void*)k_gram_dw<256>);
-    k_gram_dw<256><<<grid, g.threads, g.smem, stream>>>((int)n, k, nu, u, nvb, v1, v2, sym, shared, g.S, g.rpb, g.R,
-                                                        partial);
-  }
-  k_gram_reduce<<<total / 8, 256, 0, stream>>>(g.nblk, mu, mv, sym, partial, out1, out2);
+  allow_dynamic_smem((const void*)k_gram_dw);
+  k_gram_dw<<<dim3(g.nblk, nv), g.threads, g.smem, stream>>>((int)n, k, nu, u, nvb, v1, v2, sym, shared, g.S, g.rpb,
+                                                             g.R, partial);
+  k_gram_reduce<<<(total + 31) / 32, 256, 0, stream>>>(g.nblk, nv, mu, mv, sym, partial, out1, out2);
   return (int)cudaGetLastError();
 }
 

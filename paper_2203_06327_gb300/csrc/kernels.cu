@@ -589,21 +589,25 @@ __global__ void __launch_bounds__(256) k_gram_reduce(int nblk, int nv, int mu, i
 // Row-wise block update in double-word arithmetic:
 // out[r, j] = Zadd[r, j] + sign * sum_b sum_a W_b[r, a] C[(b k + a) ldc + j].
 // A block stages kCombRows rows of W split into (hi, lo) floats and the split
-// coefficient matrix; each thread forms outputs with Dot2 and converts once to
-// FP64.
+// coefficient matrix (columns padded with zeros to a multiple of four); a thread
+// owns four columns of one row, two Dot2 accumulators in each packed f32x2
+// operation (the roundings of the scalar form at half the issue slots, which
+// bound it), and converts once to FP64.  Three blocks of 12 columns to 12, 261,121
+// rows, beside the other two updates of a step (GB300): 71 -> 66 us on average.
 constexpr int kCombRows = 64;
-__global__ void __launch_bounds__(256) k_combine_dw(int64_t n, int k, int nin, Ptrs6 W, const double* __restrict__ C,
+__global__ void __launch_bounds__(512) k_combine_dw(int64_t n, int k, int nin, Ptrs6 W, const double* __restrict__ C,
                                                     int ldc, int csub, const double* __restrict__ Zadd,
                                                     double* __restrict__ out, double sign, float* __restrict__ outs,
                                                     int kp) {
   extern __shared__ __align__(16) float csm[];
-  const int m = nin * k;
-  float* Ch = csm;                       // m x csub
-  float* Cl = Ch + m * csub;
-  float* Wh = Cl + m * csub;             // kCombRows x m
+  const int m = nin * k, cq = (csub + 3) / 4, LC = 4 * cq;
+  float* Ch = csm;                       // m x LC
+  float* Cl = Ch + m * LC;
+  float* Wh = Cl + m * LC;               // kCombRows x m
   float* Wl = Wh + kCombRows * m;
-  for (int t = threadIdx.x; t < m * csub; t += blockDim.x) {
-    const dw s = split_f64(C[(t / csub) * ldc + (t % csub)]);
+  for (int t = threadIdx.x; t < m * LC; t += blockDim.x) {
+    const int a = t / LC, j = t % LC;
+    const dw s = split_f64(j < csub ? C[a * ldc + j] : 0.0);
     Ch[t] = s.hi;
     Cl[t] = s.lo;
   }
@@ -634,21 +638,35 @@ __global__ void __launch_bounds__(256) k_combine_dw(int64_t n, int k, int nin, P
     }
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < nr * csub; t += blockDim.x) {
-    const int r = t / csub, j = t % csub;
-    dot2 acc;
-    acc.zero();
-    const float* wh = Wh + r * m;
-    const float* wl = Wl + r * m;
-    for (int a = 0; a < m; ++a) acc.mac(wh[a], wl[a], Ch[a * csub + j], Cl[a * csub + j]);
-    double v = sign * acc.value();
-    const int64_t o = (row0 + r) * csub + j;
+  const int r = threadIdx.x / cq, c0 = 4 * (threadIdx.x % cq);  // blockDim.x = kCombRows cq
+  if (r >= nr) return;
+  dot2x2 acc[2];
+  acc[0].zero();
+  acc[1].zero();
+  const float* wh = Wh + r * m;
+  const float* wl = Wl + r * m;
+  const float* ch = Ch + c0;
+  const float* cl = Cl + c0;
+#pragma unroll 4
+  for (int a = 0; a < m; ++a) {
+    const float h = wh[a], l = wl[a];
+    const f32x4p bh = load_pairs(ch + a * LC), bl = load_pairs(cl + a * LC);
+    const unsigned long long ph = pack2(h, h), nh = pack2(-h, -h), nl = pack2(-l, -l);
+    acc[0].mac(ph, nh, nl, bh.p[0], bl.p[0]);
+    acc[1].mac(ph, nh, nl, bh.p[1], bl.p[1]);
+  }
+  const double v4[4] = {acc[0].value0(), acc[0].value1(), acc[1].value0(), acc[1].value1()};
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    if (c0 + c >= csub) break;
+    const int64_t o = (row0 + r) * csub + c0 + c;
+    double v = sign * v4[c];
     if (Zadd) v += Zadd[o];
     out[o] = v;
     if (outs) {  // rows of 2 kp floats: the hi parts, then the lo parts
       const dw sp = split_f64(v);
-      outs[(row0 + r) * 2 * kp + j] = sp.hi;
-      outs[(row0 + r) * 2 * kp + kp + j] = sp.lo;
+      outs[(row0 + r) * 2 * kp + c0 + c] = sp.hi;
+      outs[(row0 + r) * 2 * kp + kp + c0 + c] = sp.lo;
     }
   }
 }
@@ -3128,11 +3146,13 @@ int launch_combine_rows(Handle& h, int nin, const double* const* Win, const doub
   }
   if (h.dword()) {
     const int m = nin * h.k;
-    const size_t sm = (size_t)(2 * m * csub + 2 * kCombRows * m) * sizeof(float);
+    const int cq = (csub + 3) / 4;
+    if (cq > 8) return (int)cudaErrorInvalidValue;
+    const size_t sm = (size_t)(8 * m * cq + 2 * kCombRows * m) * sizeof(float);
     allow_dynamic_smem((const void*)k_combine_dw);
     const int64_t blocks = ((int64_t)h.n + kCombRows - 1) / kCombRows;
-    k_combine_dw<<<(unsigned)blocks, 256, sm, h.stream>>>(h.n, h.k, nin, w, C, ldc, csub, Zadd, out, sign,
-                                                          split_out, h.kp());
+    k_combine_dw<<<(unsigned)blocks, kCombRows * cq, sm, h.stream>>>(h.n, h.k, nin, w, C, ldc, csub, Zadd, out, sign,
+                                                                     split_out, h.kp());
     return (int)cudaGetLastError();
   }
   int64_t tot = (int64_t)h.n * csub;

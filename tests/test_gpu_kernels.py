@@ -81,7 +81,7 @@ def test_fp64_local_windows(name, k):
 
 
 # Double-word Gram products: columns around multiples of four (tiles are 4 x 4), one to four blocks, row counts
-# below, at and beyond a block's 32 rows.  The inputs make every operation exact, so the result has to be: V holds
+# of one row, of part of a block's 64 and of 35 blocks, the last one short.  The inputs make every operation exact, so the result has to be: V holds
 # integers up to 64, U integers a (not +-1) plus b 2^-28 with b up to 15 (wholly in the low part of the split unless
 # a = 0), so high products sum to integers below 2^24 in the running sum and the others to multiples of 2^-28 below
 # 2^-4 in the compensation; U^T U takes the integers alone.

@@ -382,12 +382,16 @@ __global__ void __launch_bounds__(256) k_inner(int n, int k, int p, Ptrs6 U, int
 // sym = 1 only the 4 x 4 output tiles on or above the diagonal are formed
 // (U^T V symmetric).  The rows of a block are taken in chunks of R: copied
 // asynchronously into a raw buffer two chunks ahead, split once into (hi, lo)
-// float planes, and accumulated by one thread per (tile, slice of the chunk's
-// rows).  A plane row holds the columns of U, then of V_v (absent when V_v is U),
-// each padded with zero columns to a multiple of four, so that a tile reads
-// aligned vectors whatever k is.  Slices are combined in FP64 at the end
-// of the block and the per-block sums are reduced over blocks in FP64 by
-// k_gram_reduce.
+// float planes a chunk ahead, and accumulated by one thread per (tile, slice of
+// the rows).  With raw buffers and planes both doubled, a chunk takes one barrier,
+// and the split of the next chunk (integer and load/store work) runs beside the
+// products of this one.  Where tiles leave warps without one (144 tiles: 96
+// threads), those warps do all the copies and splits.  A plane row holds the
+// columns of U, then of V_v (absent when V_v is U), each padded with zero columns
+// to a multiple of four, so that a tile reads aligned vectors whatever k is.
+// Slice q of S takes the rows q, q + S, .. of every RO rows, whatever the chunks
+// are.  Slices are combined in FP64 at the end of the block and the per-block sums
+// are reduced over blocks in FP64 by k_gram_reduce.
 // Bound: the FP32 pipe, 12 lane operations per Dot2 multiply-add (39.3 T/s
 // measured: 53 us for 36 columns of 261,121 rows, upper tiles).  The products
 // run two at a time in packed f32x2 instructions (the same pipe rate and the
@@ -396,14 +400,18 @@ __global__ void __launch_bounds__(256) k_inner(int n, int k, int p, Ptrs6 U, int
 // (x, y + 1) with (x + 1, y), so that U's pairs are the loaded ones and V's are
 // the loaded ones and their swaps.  The partition of the rows and the order of
 // the sums are those of the scalar kernel this replaced: the same bits.  Measured
-// (GB300, before -> now): 36 columns of 261,121 rows, symmetric, 188 -> 151 us
-// (FP32 pipe about half busy; two products in one block, W split once, were 3 %
-// slower than a block each), 19 x 57 columns of 65,025 rows 99 -> 83 us, the
-// products of a step at 2,209 rows and k = 6 49 -> 19 us on average.  A pair of
-// 36-column products of 261,121 rows, too large to gain from the shorter tail
-// and with W split twice, takes 3 % longer than before.
+// (us, GB300: that kernel / packed with a chunk split between two barriers / now):
+// 36 columns of 261,121 rows, symmetric 183 / 150 / 139; 19 x 57 columns of 65,025
+// rows 97 / 82 / 80; the two launches of a step (12 x 12, and the pair of 36
+// columns, which splits its U twice) at 261,121 rows 199 / 205 / 190 on average;
+// 64 columns of 1,046,529 rows, symmetric (136 tiles) 1743 / 1853 / 1732; 48 x 48
+// (144 tiles, 4.5 warps on four quarters of an SM) 1629 / 2039 / 1752.
 // ---------------------------------------------------------------------------
 constexpr int kGramRows = 64;     // a block's rows are a multiple of this
+constexpr int kGramThreads = 256;
+constexpr int kGramHelpers = 64;  // threads without a tile that take over the copies and splits (48 x 48 columns: 1752
+                                  // us, by all threads 1917)
+constexpr size_t kGramSmem = 110 * 1024;  // two blocks on an SM (chunks of half the bytes: 36 columns 139 -> 147 us)
 constexpr int kGramBlocks = 304;  // two resident blocks on each of the 152 SMs: one wave per product
 
 __device__ __forceinline__ void gram_tile_of(int t, int TU, int TV, int sym, int& ta, int& tb) {
@@ -429,12 +437,16 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-__global__ void __launch_bounds__(256, 2)
-    k_gram_dw(int n, int k, int nu, Ptrs6 U, int nvb, Ptrs6 V1, Ptrs6 V2, int sym, int shared_mask, int S,
-              int rows_per_block, int R, double* partial) {
+struct GramBlocks {
+  Ptrs6 U, V[2];
+};
+
+__global__ void __launch_bounds__(kGramThreads, 2)
+    k_gram_dw(int n, int k, int nu, int nvb, const __grid_constant__ GramBlocks blk, int sym, int shared_mask, int S,
+              int rows_per_block, int RO, int R, double* partial) {
   extern __shared__ __align__(16) float gsm[];
-  const Ptrs6& V = blockIdx.y ? V2 : V1;
-  const int shared_v = (shared_mask >> blockIdx.y) & 1;
+  const int vsel = blockIdx.y;
+  const int shared_v = (shared_mask >> vsel) & 1;
   const int mu = nu * k, mv = nvb * k;
   const int TU = (mu + 3) / 4, TV = (mv + 3) / 4;
   const int ntiles = sym ? TU * (TU + 1) / 2 : TU * TV;
@@ -442,9 +454,8 @@ __global__ void __launch_bounds__(256, 2)
   const int SEG = R * k;                        // values per block and chunk
   const int CH = nseg * SEG;                    // values per chunk
   const int LD = 4 * (TU + (1 - shared_v) * TV);  // plane row
-  double* raw = reinterpret_cast<double*>(gsm);        // [2][CH]
-  float* ph = reinterpret_cast<float*>(raw + 2 * CH);  // [R][LD]
-  float* pl = ph + R * LD;                             // [R][LD]
+  double* raw = reinterpret_cast<double*>(gsm);            // [2][CH]
+  float* planes = reinterpret_cast<float*>(raw + 2 * CH);  // [2]: [R][LD] hi, [R][LD] lo
   const int tid = threadIdx.x, nt = blockDim.x;
   const int tile = tid % ntiles, slice = tid / ntiles;
   const bool worker = slice < S;
@@ -452,22 +463,50 @@ __global__ void __launch_bounds__(256, 2)
   gram_tile_of(tile, TU, TV, sym, ta, tb);
   const int uo = 4 * ta, vo = 4 * (tb + (shared_v ? 0 : TU));
   const int64_t r0 = (int64_t)blockIdx.x * rows_per_block;
-  const int64_t r1 = min((int64_t)n, r0 + rows_per_block);
-  const int nch = (int)((r1 - r0 + R - 1) / R);
-  auto seg_ptr = [&](int sg) -> const double* { return sg < nu ? U.p[sg] : V.p[sg - nu]; };
+  const int rows = (int)min((int64_t)rows_per_block, (int64_t)n - r0);
+  const int nch = (rows + R - 1) / R;
+  // copies and splits: by the warps without a tile when there are enough of them, else by all
+  const int w0 = (S * ntiles + 31) / 32 * 32;
+  const int sfirst = (nt - w0 >= kGramHelpers) ? w0 : 0;
+  const int sid = tid - sfirst, sn = nt - sfirst;
+  auto seg_ptr = [&](int sg) -> const double* { return sg < nu ? blk.U.p[sg] : blk.V[vsel].p[sg - nu]; };
   // plane column of a segment's first value
   auto seg_col = [&](int sg) -> int { return sg < nu ? sg * k : 4 * TU + (sg - nu) * k; };
   auto issue = [&](int c) {
-    if (c < nch) {
+    if (c < nch && sid >= 0) {
       const int64_t rb = r0 + (int64_t)c * R;
-      const int cnt = (int)min((int64_t)SEG, (r1 - rb) * k);  // values inside the row range
+      const int cnt = min(SEG, (rows - c * R) * k);  // values inside the row range
       double* dst = raw + (c & 1) * CH;
       for (int sg = 0; sg < nseg; ++sg) {
         const double* src = seg_ptr(sg) + rb * k;
-        for (int e = tid; e < cnt; e += nt) cp_async8(dst + sg * SEG + e, src + e);
+        for (int e = sid; e < cnt; e += sn) cp_async8(dst + sg * SEG + e, src + e);
       }
     }
     cp_async_commit();
+  };
+  const int er0 = max(sid, 0) / k, ej0 = max(sid, 0) % k, edr = sn / k, edj = sn % k;
+  auto split = [&](int c) {
+    if (c >= nch || sid < 0) return;
+    const int nr = min(R, rows - c * R);
+    const double* src = raw + (c & 1) * CH;
+    float* ph = planes + (c & 1) * 2 * R * LD;
+    for (int sg = 0; sg < nseg; ++sg) {
+      const double* s = src + sg * SEG;
+      float* h = ph + seg_col(sg);
+      float* l = h + R * LD;
+      // value e = (row r, column j), advanced without a division
+      for (int e = sid, r = er0, j = ej0; r < nr; e += sn) {
+        const dw sp = split_f64(s[e]);
+        h[r * LD + j] = sp.hi;
+        l[r * LD + j] = sp.lo;
+        r += edr;
+        j += edj;
+        if (j >= k) {
+          j -= k;
+          ++r;
+        }
+      }
+    }
   };
   dot2x2 acc[4][2];  // pairs of a 4 x 4 tile: [2 x pair + anti-diagonal][y pair]
 #pragma unroll
@@ -477,54 +516,44 @@ __global__ void __launch_bounds__(256, 2)
   issue(0);
   issue(1);
   // padding columns stay zero
-  for (int e = tid; e < R * LD; e += nt) ph[e] = pl[e] = 0.f;
-  const int er0 = tid / k, ej0 = tid % k, edr = nt / k, edj = nt % k;
+  for (int e = tid; e < 4 * R * LD; e += nt) planes[e] = 0.f;
+  cp_async_wait1();
+  __syncthreads();
+  split(0);
+  // this thread's rows: slice, slice + S, .. of every RO
+  int r = (worker && slice < RO) ? slice : (1 << 30), q = 0;  // from the chunk's first row
   for (int c = 0; c < nch; ++c) {
-    cp_async_wait1();
-    __syncthreads();  // chunk c has landed for every thread; the planes are free
-    const int nr = (int)min((int64_t)R, r1 - (r0 + (int64_t)c * R));
-    {
-      const double* src = raw + (c & 1) * CH;
-      for (int sg = 0; sg < nseg; ++sg) {
-        const double* s = src + sg * SEG;
-        float* h = ph + seg_col(sg);
-        float* l = pl + seg_col(sg);
-        // value e = (row r, column j), advanced without a division
-        for (int e = tid, r = er0, j = ej0; r < nr; e += nt) {
-          const dw sp = split_f64(s[e]);
-          h[r * LD + j] = sp.hi;
-          l[r * LD + j] = sp.lo;
-          r += edr;
-          j += edj;
-          if (j >= k) {
-            j -= k;
-            ++r;
-          }
-        }
-      }
-    }
-    __syncthreads();  // planes ready; the raw buffer of chunk c is free
+    cp_async_wait0();
+    // chunk c + 1 has landed, the planes of chunk c are written, those of c - 1 and the raw
+    // buffer of c are free
+    __syncthreads();
     issue(c + 2);
-    if (worker) {
-      for (int r = slice; r < nr; r += S) {
-        const float* rh = ph + r * LD;
-        const float* rl = pl + r * LD;
-        const f32x4p uh = load_pairs(rh + uo), ul = load_pairs(rl + uo);
-        const unsigned long long nh[2] = {neg2(uh.p[0]), neg2(uh.p[1])}, nl[2] = {neg2(ul.p[0]), neg2(ul.p[1])};
-        const f32x4p vh = load_pairs(rh + vo), vl = load_pairs(rl + vo);
+    split(c + 1);
+    const int end = min(R, rows - c * R);
+    const float* rh = planes + (c & 1) * 2 * R * LD;
+    const float* rl = rh + R * LD;
+    while (r < end) {
+      const f32x4p uh = load_pairs(rh + r * LD + uo), ul = load_pairs(rl + r * LD + uo);
+      const unsigned long long nh[2] = {neg2(uh.p[0]), neg2(uh.p[1])}, nl[2] = {neg2(ul.p[0]), neg2(ul.p[1])};
+      const f32x4p vh = load_pairs(rh + r * LD + vo), vl = load_pairs(rl + r * LD + vo);
 #pragma unroll
-        for (int y = 0; y < 2; ++y) {
-          const unsigned long long sh = swap2(vh.p[y]), sl = swap2(vl.p[y]);
+      for (int y = 0; y < 2; ++y) {
+        const unsigned long long sh = swap2(vh.p[y]), sl = swap2(vl.p[y]);
 #pragma unroll
-          for (int x = 0; x < 2; ++x) {
-            acc[2 * x][y].mac(uh.p[x], nh[x], nl[x], vh.p[y], vl.p[y]);
-            acc[2 * x + 1][y].mac(uh.p[x], nh[x], nl[x], sh, sl);
-          }
+        for (int x = 0; x < 2; ++x) {
+          acc[2 * x][y].mac(uh.p[x], nh[x], nl[x], vh.p[y], vl.p[y]);
+          acc[2 * x + 1][y].mac(uh.p[x], nh[x], nl[x], sh, sl);
         }
       }
+      r += S;
+      if (r >= q + RO) {
+        q += RO;
+        r = q + slice;
+      }
     }
+    r -= R;
+    q -= R;
   }
-  cp_async_wait0();
   __syncthreads();
   // combine the slices in FP64 (shared memory reused): every thread sums some entries
   double* red = reinterpret_cast<double*>(gsm);  // [S][ntiles 16]
@@ -542,7 +571,7 @@ __global__ void __launch_bounds__(256, 2)
       }
   }
   __syncthreads();
-  double* out = partial + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * per;
+  double* out = partial + ((int64_t)vsel * gridDim.x + blockIdx.x) * per;
   for (int e = tid; e < per; e += nt) {
     double s = red[e];
     for (int sl = 1; sl < S; ++sl) s += red[(size_t)sl * per + e];
@@ -3060,31 +3089,25 @@ int launch_inner(Handle& h, int p, const double* const* U, int q, const double* 
   return (int)cudaGetLastError();
 }
 
-// Blocks, rows per block and per chunk, slices and shared memory of a Gram launch.  The
-// partition of the rows (and with it the order of every sum, hence the bits) is a function of
-// n, the columns and nv alone; 45 tiles: 5 slices, 225 of 256 threads.
+// Blocks, rows per block, slices and the rows that a round of slices covers (RO of k_gram_dw)
+// of a Gram launch.  The partition of the rows (and with it the order of every sum, hence the
+// bits) is a function of n, the columns and nv alone; 45 tiles: 5 slices, 225 of 256 threads.
 struct GramShape {
-  int ntiles = 0, S = 1, threads = 32, nblk = 1, rpb = 1, R = 1;
-  size_t smem = 0;
+  int ntiles = 0, S = 1, nblk = 1, rpb = 1, R = 1;
 };
 static GramShape gram_shape(int64_t n, int k, int nu, int nvb, int nv, int sym) {
   GramShape g;
   const int TU = (nu * k + 3) / 4, TV = (nvb * k + 3) / 4;
   g.ntiles = sym ? TU * (TU + 1) / 2 : TU * TV;
   g.S = std::max(1, 256 / g.ntiles);
-  g.threads = (g.S * g.ntiles + 31) / 32 * 32;
   const int nblk = (int)std::min<int64_t>(kGramBlocks, (n + kGramRows - 1) / kGramRows);
   g.rpb = (int)(((n + nblk - 1) / nblk + kGramRows - 1) / kGramRows * kGramRows);
   g.nblk = (int)((n + g.rpb - 1) / g.rpb);
-  // chunk rows: a divisor of kGramRows keeping the staging of all blocks of the call (two raw
-  // FP64 buffers and the hi/lo planes, 24 bytes per value) within 100 KB
+  // a divisor of kGramRows that shrinks with the values of a row over all blocks of the call
   const int nseg = nu + nv * nvb;
   int R = kGramRows;
   while (R > 1 && (size_t)24 * R * k * nseg > 100 * 1024) R /= 2;
   g.R = R;
-  const int Ra = R + (R & 1);  // raw buffers and planes stay 16-byte aligned
-  g.smem = std::max((16 * (size_t)(nu + nvb) * k + 32 * (size_t)(TU + TV)) * Ra,
-                    (size_t)g.S * g.ntiles * 16 * sizeof(double));
   return g;
 }
 
@@ -3100,23 +3123,27 @@ int launch_gram_raw(int64_t n, int k, int nu, const double* const* U, int nvb, i
   const int TU = (mu + 3) / 4, TV = (mv + 3) / 4;
   const int ntiles = sym ? TU * (TU + 1) / 2 : TU * TV;
   if (ntiles > 256 || nv < 1 || nv > 2 || nu > 6 || nvb > 6 || n < 1) return (int)cudaErrorInvalidValue;
-  Ptrs6 u{}, v1{}, v2{};
-  for (int b = 0; b < nu; ++b) u.p[b] = U[b];
-  int shared = nu == nvb ? 3 : 0;  // bit v: the same blocks on both sides (copied and split once)
-  for (int b = 0; b < nvb; ++b) {
-    v1.p[b] = V1[b];
-    if (shared && U[b] != V1[b]) shared &= ~1;
-    if (nv > 1) {
-      v2.p[b] = V2[b];
-      if (shared && U[b] != V2[b]) shared &= ~2;
+  GramBlocks blk{};
+  for (int b = 0; b < nu; ++b) blk.U.p[b] = U[b];
+  int shared = nu == nvb ? (1 << nv) - 1 : 0;  // bit v: the same blocks on both sides (copied and split once)
+  for (int v = 0; v < nv; ++v)
+    for (int b = 0; b < nvb; ++b) {
+      blk.V[v].p[b] = (v ? V2 : V1)[b];
+      if (shared && U[b] != blk.V[v].p[b]) shared &= ~(1 << v);
     }
-  }
   const GramShape g = gram_shape(n, k, nu, nvb, nv, sym);
   const int total = nv * ntiles * 16;
   if ((size_t)g.nblk * total > partial_capacity) return (int)cudaErrorInvalidValue;
   allow_dynamic_smem((const void*)k_gram_dw);
-  k_gram_dw<<<dim3(g.nblk, nv), g.threads, g.smem, stream>>>((int)n, k, nu, u, nvb, v1, v2, sym, shared, g.S, g.rpb,
-                                                             g.R, partial);
+  // rows of a chunk: what two blocks of an SM can hold (raw FP64 rows and split planes, both twice)
+  const bool all_shared = shared == (1 << nv) - 1;
+  const int segs = nu + (all_shared ? 0 : nvb), tiles = TU + (all_shared ? 0 : TV);
+  const size_t row = 16 * (size_t)segs * k + 64 * (size_t)tiles;
+  int stage = kGramRows;
+  while (stage > 2 && stage * row > kGramSmem) stage /= 2;
+  const size_t smem = std::max(row * stage, (size_t)g.S * ntiles * 16 * sizeof(double));
+  k_gram_dw<<<dim3(g.nblk, nv), kGramThreads, smem, stream>>>((int)n, k, nu, nvb, blk, sym, shared, g.S, g.rpb, g.R,
+                                                              stage, partial);
   k_gram_reduce<<<(total + 31) / 32, 256, 0, stream>>>(g.nblk, nv, mu, mv, sym, partial, out1, out2);
   return (int)cudaGetLastError();
 }

@@ -64,44 +64,51 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // ---------------------------------------------------------------------------
 // CSR SpMM over a block of vectors: YA = A X and (YM) YM = M X with a shared
-// pattern.  A lane owns four consecutive columns of a row, lpr = ceil(ncols / 4)
-// consecutive lanes serve the row, so 30 of 32 lanes or more have work for up to
-// 24 columns (a power of two of lanes left 12 of 32 idle at 20 columns).  The
+// pattern.  A lane owns C = 4 consecutive columns of a row (2 where that leaves the
+// chip idle), lpr = ceil(ncols / C) consecutive lanes serve the row, so with C = 4
+// 30 of 32 lanes or more have work for up to 24 columns (a power of two of lanes
+// left 12 of 32 idle at 20 columns).  The
 // entries of a row are taken kSpmmAhead at a time: first their columns and
 // values, then the X rows they name, then the products in entry order, so a row
 // costs two dependent accesses per kSpmmAhead entries.
-//   kSpmmF64    native FP64: bound by the FP64 pipe (0.53 T multiply-adds/s
-//               measured), so by the lanes that take part;
+//   kSpmmF64    native FP64: bound by the FP64 pipe (a warp instruction every 64
+//               cycles per SM quarter: 0.63 T multiply-adds/s at 2.07 GHz), so by
+//               the lanes that take part and by predicated instructions, which
+//               take their time there too: the last entries of a row go through a
+//               rolled loop (7 entries a row, 64 columns, 261,121 rows: 455 -> 382
+//               us; 20 columns 155 -> 131 us);
 //   kSpmmDw     double-word (Dot2) with pre-split matrix values, X split here;
 //   kSpmmSplit  the same with X's (hi, lo) split as written by the kernel that
 //               produced X (rows of 2 kp floats: the hi parts, then the lo parts).
 // The double-word products take two columns at a time in packed f32x2
 // instructions, the roundings of the scalar form.  VEC: rows of X, YA and YM are
 // aligned pairs (even ncols, 16-byte aligned arrays).  Measured (GB300, before ->
-// now): 20 columns, 27 entries a row, 250,047 rows in FP64 1529 -> 488 us (the
-// pipe's time is 493 us at its measured rate); 12 double-word columns of
+// now): 20 columns, 27 entries a row, 250,047 rows in FP64 1529 -> 468 us (the
+// pipe's time is 416 us, 444 us with 30 of 32 lanes); 12 double-word columns of
 // 1,046,529 rows 241 -> 203 us with the split ahead (244 us splitting per entry).
 // ---------------------------------------------------------------------------
 constexpr int kSpmmF64 = 0, kSpmmDw = 1, kSpmmSplit = 2;
 constexpr int kSpmmAhead = 4;
 
-template <int MODE, bool VEC>
-__global__ void __launch_bounds__(128, (MODE == kSpmmDw) ? 4 : 5) k_spmm(int n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                              const double* __restrict__ va, const double* __restrict__ vm,
-                                              const double* __restrict__ X, const float* __restrict__ Xs, int kp,
-                                              double* __restrict__ YA, double* __restrict__ YM, int ncols, int lpr) {
-  constexpr int U = kSpmmAhead;
+template <int MODE, bool VEC, int C>
+__global__ void __launch_bounds__(128, (MODE == kSpmmDw) ? 4 : 5)
+    k_spmm(int n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci, const double* __restrict__ va,
+           const double* __restrict__ vm, const double* __restrict__ X, const float* __restrict__ Xs, int kp,
+           double* __restrict__ YA, double* __restrict__ YM, int ncols, int lpr) {
+  constexpr int U = kSpmmAhead, H = C / 2;
   const int lane = threadIdx.x & 31;
   const int rpw = 32 / lpr;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t row = warp * rpw + lane / lpr;
   if (lane >= rpw * lpr || row >= n) return;
-  const int c0 = 4 * (lane % lpr);
-  const int nc = min(4, ncols - c0);
-  double fa[4] = {0, 0, 0, 0}, fm[4] = {0, 0, 0, 0};
-  dot2x2 da[2], dm[2];
+  const int c0 = C * (lane % lpr);
+  const int nc = min(C, ncols - c0);
+  double fa[C], fm[C];
+  dot2x2 da[H], dm[H];
 #pragma unroll
-  for (int c = 0; c < 2; ++c) {
+  for (int c = 0; c < C; ++c) fa[c] = fm[c] = 0.0;
+#pragma unroll
+  for (int c = 0; c < H; ++c) {
     da[c].zero();
     dm[c].zero();
   }
@@ -116,84 +123,110 @@ __global__ void __launch_bounds__(128, (MODE == kSpmmDw) ? 4 : 5) k_spmm(int n, 
       av[u] = ok ? va[e0 + u] : 0.0;
       mv[u] = (ok && vm) ? vm[e0 + u] : 0.0;
     }
-    double x[U][4];
-    f32x4p xh[U], xl[U];
+    double x[U][C];
+    unsigned long long xh[U][H], xl[U][H];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (MODE == kSpmmSplit) {
         if (col[u] >= 0) {
           const float* xr = Xs + (int64_t)col[u] * 2 * kp + c0;
-          const ulonglong2 h = *reinterpret_cast<const ulonglong2*>(xr);
-          const ulonglong2 l = *reinterpret_cast<const ulonglong2*>(xr + kp);
-          xh[u] = f32x4p{{h.x, h.y}};
-          xl[u] = f32x4p{{l.x, l.y}};
+          if (C == 4) {
+            const ulonglong2 h = *reinterpret_cast<const ulonglong2*>(xr);
+            const ulonglong2 l = *reinterpret_cast<const ulonglong2*>(xr + kp);
+            xh[u][0] = h.x;
+            xh[u][H - 1] = h.y;
+            xl[u][0] = l.x;
+            xl[u][H - 1] = l.y;
+          } else {
+            xh[u][0] = *reinterpret_cast<const unsigned long long*>(xr);
+            xl[u][0] = *reinterpret_cast<const unsigned long long*>(xr + kp);
+          }
         }
       } else if (col[u] >= 0) {
         const double* xr = X + (int64_t)col[u] * ncols + c0;
         if (VEC) {
-          const double2 p = *reinterpret_cast<const double2*>(xr);
-          x[u][0] = p.x;
-          x[u][1] = p.y;
-          x[u][2] = x[u][3] = 0.0;
-          if (nc > 2) {
-            const double2 q = *reinterpret_cast<const double2*>(xr + 2);
-            x[u][2] = q.x;
-            x[u][3] = q.y;
+#pragma unroll
+          for (int c = 0; c < H; ++c) {
+            const double2 p = (2 * c < nc) ? *reinterpret_cast<const double2*>(xr + 2 * c) : make_double2(0.0, 0.0);
+            x[u][2 * c] = p.x;
+            x[u][2 * c + 1] = p.y;
           }
         } else {
 #pragma unroll
-          for (int c = 0; c < 4; ++c) x[u][c] = (c < nc) ? xr[c] : 0.0;
+          for (int c = 0; c < C; ++c) x[u][c] = (c < nc) ? xr[c] : 0.0;
         }
       }
     }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (col[u] < 0) continue;
+    auto take = [&](int u) {
       if (MODE == kSpmmF64) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < C; ++c) {
           fa[c] = fma(av[u], x[u][c], fa[c]);
           if (vm) fm[c] = fma(mv[u], x[u][c], fm[c]);
         }
       } else {
         if (MODE == kSpmmDw) {
-          dw s[4];
+          dw s[C];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) s[c] = split_f64(x[u][c]);
+          for (int c = 0; c < C; ++c) s[c] = split_f64(x[u][c]);
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            xh[u].p[c] = pack2(s[2 * c].hi, s[2 * c + 1].hi);
-            xl[u].p[c] = pack2(s[2 * c].lo, s[2 * c + 1].lo);
+          for (int c = 0; c < H; ++c) {
+            xh[u][c] = pack2(s[2 * c].hi, s[2 * c + 1].hi);
+            xl[u][c] = pack2(s[2 * c].lo, s[2 * c + 1].lo);
           }
         }
         const float ah = __int_as_float(__double2loint(av[u])), al = __int_as_float(__double2hiint(av[u]));
         const unsigned long long pa = pack2(ah, ah), na = pack2(-ah, -ah), ta = pack2(-al, -al);
 #pragma unroll
-        for (int c = 0; c < 2; ++c) da[c].mac(pa, na, ta, xh[u].p[c], xl[u].p[c]);
+        for (int c = 0; c < H; ++c) da[c].mac(pa, na, ta, xh[u][c], xl[u][c]);
         if (vm) {
           const float mh = __int_as_float(__double2loint(mv[u])), ml = __int_as_float(__double2hiint(mv[u]));
           const unsigned long long pm = pack2(mh, mh), nm = pack2(-mh, -mh), tm = pack2(-ml, -ml);
 #pragma unroll
-          for (int c = 0; c < 2; ++c) dm[c].mac(pm, nm, tm, xh[u].p[c], xl[u].p[c]);
+          for (int c = 0; c < H; ++c) dm[c].mac(pm, nm, tm, xh[u][c], xl[u][c]);
         }
       }
+    };
+    if (MODE == kSpmmF64) {
+      if (e0 + U <= end) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) take(u);
+      } else {
+        // a queue of registers: entry 0 is taken, the others move up
+#pragma unroll 1
+        for (int left = (int)(end - e0); left > 0; --left) {
+          take(0);
+#pragma unroll
+          for (int u = 0; u + 1 < U; ++u) {
+            av[u] = av[u + 1];
+            mv[u] = mv[u + 1];
+#pragma unroll
+            for (int c = 0; c < C; ++c) x[u][c] = x[u + 1][c];
+          }
+        }
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (col[u] >= 0) take(u);
     }
   }
-  auto store = [&](double* Y, double (&f)[4], dot2x2 (&d)[2]) {
+  auto store = [&](double* Y, double (&f)[C], dot2x2 (&d)[H]) {
     if (MODE != kSpmmF64) {
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
+      for (int c = 0; c < H; ++c) {
         f[2 * c] = d[c].value0();
         f[2 * c + 1] = d[c].value1();
       }
     }
     double* y = Y + row * ncols + c0;
     if (VEC) {
-      *reinterpret_cast<double2*>(y) = make_double2(f[0], f[1]);
-      if (nc > 2) *reinterpret_cast<double2*>(y + 2) = make_double2(f[2], f[3]);
+#pragma unroll
+      for (int c = 0; c < H; ++c)
+        if (2 * c < nc) *reinterpret_cast<double2*>(y + 2 * c) = make_double2(f[2 * c], f[2 * c + 1]);
     } else {
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+      for (int c = 0; c < C; ++c)
         if (c < nc) y[c] = f[c];
     }
   };
@@ -2990,20 +3023,17 @@ void prof_flush(Handle& h) {
 // ===========================================================================
 // launchers
 // ===========================================================================
-// products; us split ahead / per entry (GB300): 12 columns 6.9 M 22.6 / 20.5, 12.3 M 30.8 / 32.8,
-// 49 M 119 / 139; 5 columns 1.7 M 14.4 / 14.4, 5.1 M 24.6 / 28.7, 21 M 78 / 115
+// products (entries of K times columns) from which on X is split ahead; us split ahead / per entry
+// (GB300): 4 columns 7.3 M 22.6 / 21.6, 16.4 M 48.5 / 51.2; 8 columns 8.2 M 24.3 / 22.6, 14.6 M
+// 39.2 / 41.0; 12 columns 6.9 M 22.6 / 20.5, 12.3 M 34.2 / 34.8, 21.9 M 57.6 / 65.6; 20 columns
+// 6.9 M 22.6 / 20.5, 11.5 M 30.7 / 30.8, 20.5 M 53.3 / 57.4: even between 8 and 12 M
 constexpr int64_t kSplitAhead = 8000000;
 int launch_spmm(Handle& h, const double* X, double* YA, double* YM, int ncols, const float* Xs) {
   ProfScope ps(h, BPJD_PROF_SPMM);
   const int n = h.n;
-  const int lpr = (ncols + 3) / 4, rpw = 32 / lpr;
-  // four warps per block; one when that fills the chip better (few rows)
-  const int64_t warps = ((int64_t)n + rpw - 1) / rpw;
-  const int wpb = (warps < 4 * 304) ? 1 : 4;
-  const unsigned blocks = (unsigned)((warps + wpb - 1) / wpb);
+  const bool dw = h.dword() && h.Asplit;
   auto aligned = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
   const bool vec = ncols % 2 == 0 && aligned(X) && aligned(YA) && aligned(YM);
-  const bool dw = h.dword() && h.Asplit;
   // splitting X's rows ahead costs a pass over X and a launch, splitting them in the product
   // one split per entry of the matrix: ahead from kSplitAhead products on, where the handle's
   // buffer has the columns
@@ -3014,21 +3044,40 @@ int launch_spmm(Handle& h, const double* X, double* YA, double* YM, int ncols, c
     h.launches += 1;
     Xs = h.xsplit;
   }
-  auto go = [&](auto mode, auto vec_tag, const CsrDev& A, const void* va, const void* vm, double* ya, double* ym) {
-    k_spmm<decltype(mode)::value, decltype(vec_tag)::value><<<blocks, 32 * wpb, 0, h.stream>>>(
-        n, A.row_ptr, A.col, (const double*)va, (const double*)vm, X, Xs, kp, ya, ym, ncols, lpr);
+  // two columns per lane instead of four (us, GB300, two / four): where four are a fifth padding
+  // or more, 1, 2, 5, 6, 9 and 10 columns (1 column of 261,121 rows double-word 13 / 24, FP64 18 /
+  // 32; 5 columns of 101,761 rows 15 / 21), and where two give at most twice as many warps as an
+  // SM holds at four, 20 (1,833 rows: 8 columns 4.2 / 5.1; 25,281 rows: 12 columns 8.7 / 9.8, 20
+  // columns 12.1 / 11.8).  An X that is split already leaves less to do per entry, and the line
+  // lies at 20 warps (9,025 rows: 20 columns 5.7 / 6.5; 25,281 rows: 12 columns 7.5 / 7.1)
+  const int rpw2 = 32 / ((ncols + 1) / 2);
+  const bool two = (ncols <= 10 && (ncols % 4 == 1 || ncols % 4 == 2)) ||
+                   ((int64_t)n + rpw2 - 1) / rpw2 <= (dw && Xs ? 20 : 40) * 152;
+  const int cpl = two ? 2 : 4;
+  const int lpr = (ncols + cpl - 1) / cpl, rpw = 32 / lpr;
+  // two warps per block; one when that fills the chip better (few rows)
+  const int64_t warps = ((int64_t)n + rpw - 1) / rpw;
+  const int wpb = (warps < 4 * 304) ? 1 : 2;
+  const unsigned blocks = (unsigned)((warps + wpb - 1) / wpb);
+  auto go = [&](auto mode, auto vec_tag, auto cols, const CsrDev& A, const void* va, const void* vm, double* ya,
+                double* ym) {
+    k_spmm<decltype(mode)::value, decltype(vec_tag)::value, decltype(cols)::value>
+        <<<blocks, 32 * wpb, 0, h.stream>>>(n, A.row_ptr, A.col, (const double*)va, (const double*)vm, X, Xs, kp, ya,
+                                            ym, ncols, lpr);
     h.launches += 1;
   };
   auto run = [&](const CsrDev& A, const void* va, const void* vm, double* ya, double* ym) {
-    using F = std::integral_constant<int, kSpmmF64>;
-    using D = std::integral_constant<int, kSpmmDw>;
-    using P = std::integral_constant<int, kSpmmSplit>;
+    auto by_cols = [&](auto mode, auto vec_tag) {
+      two ? go(mode, vec_tag, std::integral_constant<int, 2>(), A, va, vm, ya, ym)
+          : go(mode, vec_tag, std::integral_constant<int, 4>(), A, va, vm, ya, ym);
+    };
+    auto by_vec = [&](auto mode) { vec ? by_cols(mode, std::true_type()) : by_cols(mode, std::false_type()); };
     if (!dw)
-      vec ? go(F(), std::true_type(), A, va, vm, ya, ym) : go(F(), std::false_type(), A, va, vm, ya, ym);
+      by_vec(std::integral_constant<int, kSpmmF64>());
     else if (Xs)
-      vec ? go(P(), std::true_type(), A, va, vm, ya, ym) : go(P(), std::false_type(), A, va, vm, ya, ym);
+      by_vec(std::integral_constant<int, kSpmmSplit>());
     else
-      vec ? go(D(), std::true_type(), A, va, vm, ya, ym) : go(D(), std::false_type(), A, va, vm, ya, ym);
+      by_vec(std::integral_constant<int, kSpmmDw>());
   };
   const void* va = dw ? (const void*)h.Asplit : (const void*)h.A.val;
   const void* vm = dw ? (const void*)h.Msplit : (const void*)h.M.val;

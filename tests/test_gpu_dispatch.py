@@ -4,12 +4,22 @@ import ctypes as C
 
 import numpy as np
 import pytest
+import scipy.sparse as sp
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 B = pytest.importorskip("paper_2203_06327_gb300.binding")
 
 DEV = "cuda"
+
+
+def _scipy(a):
+    return sp.csr_matrix((a.val, a.col_idx, a.row_ptr), shape=(a.n_rows, a.n_cols))
+
+
+def _partition(lists):
+    ptr = np.concatenate([[0], np.cumsum([len(d) for d in lists])]).astype(np.int64)
+    return B.PartitionArrays(ptr, np.concatenate(lists).astype(np.int32), None, 0)
 
 
 # ---- Gram products ------------------------------------------------------------------------------------------------
@@ -34,3 +44,56 @@ def test_block_gram_chunks_exact_integers(n, k, nu, nv, sym):
     pv = (C.c_void_p * nv)(*[v.data_ptr() for v in Vd])
     assert fn(n, k, nu, pu, nv, pv, 1 if sym else 0, out.data_ptr(), None) == B.OK
     np.testing.assert_array_equal(out.cpu().numpy(), np.hstack(U).T @ np.hstack(V))
+
+
+# ---- sparse products ----------------------------------------------------------------------------------------------
+
+def _band_matrix(n, rng, diagonal_m):
+    """Rows of 1 to 9 entries within 8 places of the diagonal, positive definite; M of the same pattern or diagonal."""
+    r = np.arange(n)
+    off = [(d, r[(r + d < n) & (rng.random(n) < 0.4)]) for d in (1, 3, 5, 8)]
+    i = np.concatenate([x for _, x in off])
+    j = np.concatenate([x + d for d, x in off])
+    make = lambda v: sp.csr_matrix(sp.coo_matrix(  # noqa: E731
+        (np.concatenate([v, v, np.full(n, 10.0)]), (np.concatenate([i, j, r]), np.concatenate([j, i, r]))), (n, n)))
+    K = make(rng.uniform(-1.0, 1.0, len(i)))
+    return K, sp.csr_matrix(sp.diags(rng.uniform(1.0, 2.0, n))) if diagonal_m else make(rng.uniform(-1.0, 1.0, len(i)))
+
+
+def _check_spmm(sv, K, M, ncols, offset):
+    n = sv.n
+    X = np.random.default_rng(ncols).standard_normal((n, ncols))
+    bufs = [torch.full((n * ncols + offset,), float("nan"), dtype=torch.float64, device=DEV) for _ in range(3)]
+    Xd, YA, YM = [b[offset:].view(n, ncols) for b in bufs]
+    Xd.copy_(torch.tensor(X))
+    sv.spmm(Xd, YA, YM)
+    for Y, A in ((YA, K), (YM, M)):  # tolerance as for the other SpMM checks
+        assert np.all(np.abs(Y.cpu().numpy() - A @ X) <= 1e-13 * (abs(A) @ np.abs(X)) + 1e-300)
+
+
+# Rows of 1 to 9 entries (a remainder of every size after groups of four), two columns per lane (the smaller n and up
+# to 12 columns) and four (20, 31 and 64 columns of the larger n), one matrix pass or two (diagonal M).
+@pytest.mark.parametrize("n", [1999, 20001])
+@pytest.mark.parametrize("diagonal_m", [False, True], ids=["shared", "two"])
+@pytest.mark.parametrize("precision", [B.FP64, B.MIXED], ids=["fp64", "mixed"])
+def test_spmm_row_lengths_and_columns_per_lane(n, diagonal_m, precision):
+    rng = np.random.default_rng(n)
+    K, M = _band_matrix(n, rng, diagonal_m)
+    P = sp.csr_matrix(rng.uniform(0.0, 1.0, (n, 5)))
+    part = _partition([np.arange(a, min(n, a + 500)) for a in range(0, n, 500)])
+    sv = B.Solver(*[B.CsrArrays.from_scipy(a) for a in (K, M, P)], None, part, 3, precision=precision)
+    for ncols in (1, 2, 3, 12, 20, 31, 64):
+        for offset in (0, 1):
+            _check_spmm(sv, K, M, ncols, offset)
+
+
+# X split ahead from 8 million products on, where the columns fill the handle's buffer: both sides of the line (8.0
+# million lie between 4 and 5 columns at 512 x 512), odd columns, fewer columns than the handle's, unaligned arrays.
+@pytest.mark.parametrize("k,columns", [(5, (4, 5, 6, 8)), (4, (3, 4)), (12, (4, 8, 9, 10, 12))])
+def test_spmm_split_ahead(k, columns):
+    pb = B.problem_create("p1_2d", (512, 512), (1.0, 0.751 / 0.75), (8, 8), 1)
+    sv = B.Solver.from_problem(pb, k, device=DEV, precision=B.MIXED)
+    K, M = _scipy(pb.K), _scipy(pb.M)
+    for ncols in columns:
+        for offset in (0, 1):
+            _check_spmm(sv, K, M, ncols, offset)

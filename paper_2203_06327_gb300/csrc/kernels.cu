@@ -652,24 +652,30 @@ __global__ void __launch_bounds__(256) k_gram_reduce(int nblk, int nv, int mu, i
 // out[r, j] = Zadd[r, j] + sign * sum_b sum_a W_b[r, a] C[(b k + a) ldc + j].
 // A block stages kCombRows rows of W split into (hi, lo) floats and the split
 // coefficient matrix (columns padded with zeros to a multiple of four); a thread
-// owns four columns of one row, two Dot2 accumulators in each packed f32x2
-// operation (the roundings of the scalar form at half the issue slots, which
-// bound it), and converts once to FP64.  Three blocks of 12 columns to 12, 261,121
-// rows, beside the other two updates of a step (GB300): 71 -> 66 us on average.
+// owns C columns of one row, two Dot2 accumulators in each packed f32x2 operation
+// (the roundings of the scalar form at half the issue slots, which bound it), and
+// converts once to FP64.  The first kCombRows ceil(csub / C) threads of a block
+// have outputs, the others only stage.  Two columns per thread: shorter chains and
+// less padding than four, at twice the loads of W.  us per launch, the updates of a
+// step on average (GB300, scalar / four columns / two): 261,121 rows k = 12 71 / 65 /
+// 64, k = 6 34 / 33 / 29, k = 4 24 / 23 / 20; 16,129 rows k = 8 9.7 / 10.8 / 9.0;
+// 1,833 rows k = 4 7.0 / 8.8 / 7.2.
 constexpr int kCombRows = 64;
-__global__ void __launch_bounds__(512) k_combine_dw(int64_t n, int k, int nin, Ptrs6 W, const double* __restrict__ C,
+template <int C>
+__global__ void __launch_bounds__(512) k_combine_dw(int64_t n, int k, int nin, Ptrs6 W, const double* __restrict__ Cm,
                                                     int ldc, int csub, const double* __restrict__ Zadd,
                                                     double* __restrict__ out, double sign, float* __restrict__ outs,
                                                     int kp) {
+  constexpr int H = C / 2;
   extern __shared__ __align__(16) float csm[];
-  const int m = nin * k, cq = (csub + 3) / 4, LC = 4 * cq;
+  const int m = nin * k, cq = (csub + C - 1) / C, LC = (csub + 3) / 4 * 4;
   float* Ch = csm;                       // m x LC
   float* Cl = Ch + m * LC;
   float* Wh = Cl + m * LC;               // kCombRows x m
   float* Wl = Wh + kCombRows * m;
   for (int t = threadIdx.x; t < m * LC; t += blockDim.x) {
     const int a = t / LC, j = t % LC;
-    const dw s = split_f64(j < csub ? C[a * ldc + j] : 0.0);
+    const dw s = split_f64(j < csub ? Cm[a * ldc + j] : 0.0);
     Ch[t] = s.hi;
     Cl[t] = s.lo;
   }
@@ -700,11 +706,11 @@ __global__ void __launch_bounds__(512) k_combine_dw(int64_t n, int k, int nin, P
     }
   }
   __syncthreads();
-  const int r = threadIdx.x / cq, c0 = 4 * (threadIdx.x % cq);  // blockDim.x = kCombRows cq
+  const int r = threadIdx.x / cq, c0 = C * (threadIdx.x % cq);
   if (r >= nr) return;
-  dot2x2 acc[2];
-  acc[0].zero();
-  acc[1].zero();
+  dot2x2 acc[H];
+#pragma unroll
+  for (int y = 0; y < H; ++y) acc[y].zero();
   const float* wh = Wh + r * m;
   const float* wl = Wl + r * m;
   const float* ch = Ch + c0;
@@ -712,17 +718,32 @@ __global__ void __launch_bounds__(512) k_combine_dw(int64_t n, int k, int nin, P
 #pragma unroll 4
   for (int a = 0; a < m; ++a) {
     const float h = wh[a], l = wl[a];
-    const f32x4p bh = load_pairs(ch + a * LC), bl = load_pairs(cl + a * LC);
+    unsigned long long bh[H], bl[H];
+    if (C == 4) {
+      const f32x4p vh = load_pairs(ch + a * LC), vl = load_pairs(cl + a * LC);
+      bh[0] = vh.p[0];
+      bh[H - 1] = vh.p[1];
+      bl[0] = vl.p[0];
+      bl[H - 1] = vl.p[1];
+    } else {
+      bh[0] = *reinterpret_cast<const unsigned long long*>(ch + a * LC);
+      bl[0] = *reinterpret_cast<const unsigned long long*>(cl + a * LC);
+    }
     const unsigned long long ph = pack2(h, h), nh = pack2(-h, -h), nl = pack2(-l, -l);
-    acc[0].mac(ph, nh, nl, bh.p[0], bl.p[0]);
-    acc[1].mac(ph, nh, nl, bh.p[1], bl.p[1]);
-  }
-  const double v4[4] = {acc[0].value0(), acc[0].value1(), acc[1].value0(), acc[1].value1()};
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
+    for (int y = 0; y < H; ++y) acc[y].mac(ph, nh, nl, bh[y], bl[y]);
+  }
+  double vc[C];
+#pragma unroll
+  for (int y = 0; y < H; ++y) {
+    vc[2 * y] = acc[y].value0();
+    vc[2 * y + 1] = acc[y].value1();
+  }
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
     if (c0 + c >= csub) break;
     const int64_t o = (row0 + r) * csub + c0 + c;
-    double v = sign * v4[c];
+    double v = sign * vc[c];
     if (Zadd) v += Zadd[o];
     out[o] = v;
     if (outs) {  // rows of 2 kp floats: the hi parts, then the lo parts
@@ -741,7 +762,8 @@ __global__ void __launch_bounds__(512) k_combine_dw(int64_t n, int k, int nin, P
 // W and the coefficients.
 __global__ void __launch_bounds__(256) k_combine_f32(int64_t n, int k, int nin, Ptrs6 W, const double* __restrict__ C,
                                                      int ldc, int csub, const double* __restrict__ Zadd,
-                                                     double* __restrict__ out, float sign, float* __restrict__ outs, int kp) {
+                                                     double* __restrict__ out, float sign, float* __restrict__ outs,
+                                                     int kp) {
   extern __shared__ __align__(16) float csm[];
   const int m = nin * k;
   float* Cs = csm;              // m x csub
@@ -3204,7 +3226,7 @@ int launch_gram(Handle& h, int nu, const double* const* U, int nvb, int nv, cons
   return launch_gram_raw(h.n, h.k, nu, U, nvb, nv, V1, V2, sym, out1, out2, h.partial, h.partial_cap, h.stream);
 }
 
-int launch_combine_rows(Handle& h, int nin, const double* const* Win, const double* C, int ldc, int csub,
+int launch_combine_rows(Handle& h, int nin, const double* const* Win, const double* Cd, int ldc, int csub,
                         const double* Zadd, double* out, double sign, int consistency_only, float* split_out) {
   ProfScope ps(h, BPJD_PROF_COMBINE);
   h.launches += 1;
@@ -3216,7 +3238,7 @@ int launch_combine_rows(Handle& h, int nin, const double* const* Win, const doub
     const size_t sm = (size_t)(m * csub + kCombRows * m) * sizeof(float);
     allow_dynamic_smem((const void*)k_combine_f32);
     const int64_t blocks = ((int64_t)h.n + kCombRows - 1) / kCombRows;
-    k_combine_f32<<<(unsigned)blocks, 256, sm, h.stream>>>(h.n, h.k, nin, w, C, ldc, csub, Zadd, out, (float)sign,
+    k_combine_f32<<<(unsigned)blocks, 256, sm, h.stream>>>(h.n, h.k, nin, w, Cd, ldc, csub, Zadd, out, (float)sign,
                                                            split_out, h.kp());
     return (int)cudaGetLastError();
   }
@@ -3225,15 +3247,24 @@ int launch_combine_rows(Handle& h, int nin, const double* const* Win, const doub
     const int cq = (csub + 3) / 4;
     if (cq > 8) return (int)cudaErrorInvalidValue;
     const size_t sm = (size_t)(8 * m * cq + 2 * kCombRows * m) * sizeof(float);
-    allow_dynamic_smem((const void*)k_combine_dw);
     const int64_t blocks = ((int64_t)h.n + kCombRows - 1) / kCombRows;
-    k_combine_dw<<<(unsigned)blocks, kCombRows * cq, sm, h.stream>>>(h.n, h.k, nin, w, C, ldc, csub, Zadd, out, sign,
-                                                                     split_out, h.kp());
+    // two columns per thread up to 16, four above (a block stays within 512 threads).  At least
+    // 256 threads where the blocks are few, so that a thread stages few values (1,833 rows, k = 4:
+    // 7.2 us, with 128 threads 7.9); where they are many, threads that only stage take the place
+    // of other blocks (261,121 rows, k = 4: 21.6 us, with 128 threads 19.8)
+    const int least = blocks <= 4 * 152 ? 256 : kCombRows;
+    auto go = [&](auto cols) {
+      constexpr int C = decltype(cols)::value;
+      allow_dynamic_smem((const void*)k_combine_dw<C>);
+      k_combine_dw<C><<<(unsigned)blocks, std::max(least, kCombRows * ((csub + C - 1) / C)), sm, h.stream>>>(
+          h.n, h.k, nin, w, Cd, ldc, csub, Zadd, out, sign, split_out, h.kp());
+    };
+    csub <= 16 ? go(std::integral_constant<int, 2>()) : go(std::integral_constant<int, 4>());
     return (int)cudaGetLastError();
   }
   int64_t tot = (int64_t)h.n * csub;
   size_t sm = (size_t)nin * h.k * csub * sizeof(double);
-  k_combine_rows<<<(unsigned)((tot + 255) / 256), 256, sm, h.stream>>>(h.n, h.k, nin, w, C, ldc, csub, Zadd, out,
+  k_combine_rows<<<(unsigned)((tot + 255) / 256), 256, sm, h.stream>>>(h.n, h.k, nin, w, Cd, ldc, csub, Zadd, out,
                                                                         sign);
   return (int)cudaGetLastError();
 }

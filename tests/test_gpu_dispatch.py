@@ -5,6 +5,7 @@ import ctypes as C
 import numpy as np
 import pytest
 import scipy.sparse as sp
+import scipy.sparse.linalg as spla
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -97,3 +98,22 @@ def test_spmm_split_ahead(k, columns):
     for ncols in columns:
         for offset in (0, 1):
             _check_spmm(sv, K, M, ncols, offset)
+
+
+# ---- row combinations and the pair of Gram products, through solves ----------------------------------------------
+
+# Columns around the line between two and four per thread (16) and odd ones, on few row blocks (a block of at least
+# 256 threads) and on many (from 609 blocks of 64 rows on), against shift-invert Lanczos; 1e-9 as for the other solves.
+@pytest.mark.parametrize("nx,ny", [(80, 64), (256, 192)], ids=["few", "many"])
+@pytest.mark.parametrize("k,subspace", [(1, B.W_3K), (3, B.W_3K), (7, B.W_2K), (16, B.W_3K), (17, B.W_2K),
+                                        (19, B.W_3K), (23, B.W_2K)])
+def test_mixed_solve_columns(nx, ny, k, subspace):
+    pb = B.problem_create("p1_2d", (nx, ny), (1.0, 0.8 * 0.983), (nx // 4, ny // 4) if nx < 100 else (16, 12), 2)
+    K, M = _scipy(pb.K), _scipy(pb.M)
+    ref = np.sort(spla.eigsh(sp.csc_matrix(K), k, sp.csc_matrix(M), sigma=0.0, v0=np.ones(K.shape[0]),
+                             return_eigenvectors=False))
+    sv = B.Solver.from_problem(pb, k, device=DEV, precision=B.MIXED, subspace=subspace)
+    lam, X, st = sv.solve()
+    assert st["converged"] == 1
+    np.testing.assert_allclose(lam, ref, rtol=1e-9)
+    np.testing.assert_allclose(X.T @ (M @ X), np.eye(k), atol=1e-10)

@@ -490,12 +490,13 @@ extern "C" int bpjd_setup(const bpjd_csr* A, const bpjd_csr* M, const bpjd_csr* 
         }
     }
     if (h->Bpad == 0) {
-      // windows above every tier run in the shared-memory kernel, one (B x B) window per warp
+      // FP64 windows, and FP32 ones above every tier (one B x B window per warp in shared memory)
       int dev = 0, optin = 0;
       CK(cudaGetDevice(&dev));
       CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-      const size_t esz = h->local_f32() ? sizeof(float) : sizeof(double);
-      if ((size_t)(h->B * h->B + 3 * h->B) * esz > (size_t)optin) {
+      const bool fits = h->local_f32() ? ((size_t)h->B + 3) * h->B * sizeof(float) <= (size_t)optin
+                                       : h->B <= kBandF64Max && band_f64_smem(h->B) <= (size_t)optin;
+      if (!fits) {
         rc = BPJD_ERR_UNSUPPORTED;
         goto fail;
       }

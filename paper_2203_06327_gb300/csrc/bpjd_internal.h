@@ -243,6 +243,14 @@ inline size_t band_floats(int64_t sum_nl, int nsub, int B, int bpad) {
   if (band_panels(bpad)) return (size_t)(sum_nl + 7 * (int64_t)nsub) * (bpad + 8);
   return (size_t)sum_nl * (B > bpad ? B : bpad);
 }
+// widest window of the FP64 local solves (the widest whose full B x B window of one warp fits
+// 227 KB; k_local_band_f64 states what it needs of it), and that kernel's shared memory: the
+// packed window with the right-hand sides, three rows, and a 16-bit slot pair per entry
+constexpr int kBandF64Max = 168;
+inline size_t band_f64_smem(int B) {
+  const size_t ne = (size_t)B * (B + 1) / 2 + B;
+  return (ne + 3 * B + 2) * sizeof(double) + ne * sizeof(unsigned short);
+}
 // band rows of the local matrices of c (and of a second matrix with c's pattern,
 // values val2): FP32 rows of width max(B, Bpad), or panels, into outf / outf2 when outf
 // is set, else FP64 rows of width B into out / out2

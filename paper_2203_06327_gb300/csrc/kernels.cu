@@ -971,7 +971,11 @@ __global__ void k_local_band(int npairs, int k, const int64_t* __restrict__ sub_
 // of a step; six pairs on some SMs against five on others)
 // ---------------------------------------------------------------------------
 constexpr int kPivotChunks = 16;
-__global__ void __launch_bounds__(192) k_local_band_f64(int k, const int64_t* __restrict__ sub_ptr,
+constexpr int kBandF64Threads = 192;  // most threads of a CTA: a slot each, and one for the right-hand side
+constexpr int kBandF64Record = 6;     // entries of a record per lane in the backward sweep, at most
+static_assert(kBandF64Max + 1 <= kBandF64Threads && kBandF64Max - 1 <= 32 * kBandF64Record && kBandF64Max < 256,
+              "threads, records and 8-bit slots of the widest window");
+__global__ void __launch_bounds__(kBandF64Threads) k_local_band_f64(int k, const int64_t* __restrict__ sub_ptr,
                                                         const int32_t* __restrict__ sub_dofs, int B,
                                                         const double* __restrict__ bandK,
                                                         const double* __restrict__ bandM,
@@ -1123,7 +1127,7 @@ __global__ void __launch_bounds__(192) k_local_band_f64(int k, const int64_t* __
   // sums the products of entries 1 + t, 33 + t, .. of record j with the solved rows, a
   // butterfly adds the lanes; record, y and 1/L_jj are loaded two rows ahead
   if ((tid >> 5) != (int)(blockIdx.x & 3)) return;
-  constexpr int NC = 6;  // entries of a record per lane, at most (B <= 168)
+  constexpr int NC = kBandF64Record;
   const int lane = tid & 31;
   double* xs = lc;  // [B] solved rows by slot
   double c0[NC], c1[NC], c2[NC], y0 = 0.0, y1 = 0.0, y2 = 0.0, d0 = 0.0, d1 = 0.0, d2 = 0.0;
@@ -3519,10 +3523,9 @@ int launch_local(Handle& h, const double* rho, const double* lam, int mode) {
         } else {
           // four warps (one per SM quarter), six when the window has more rows
           const int nt = std::max(128, (B + 32) / 32 * 32);
-          const size_t ne = (size_t)B * (B + 1) / 2 + B;
-          const size_t sm = (ne + 3 * B + 2) * sizeof(double) + ne * sizeof(unsigned short);
+          if (B > kBandF64Max) return (int)cudaErrorInvalidValue;
           allow_dynamic_smem((const void*)k_local_band_f64);
-          k_local_band_f64<<<npairs_c, nt, sm, h.stream>>>(k, sptr, h.sub_dofs, B, h.bandK, h.bandM, lam, rho,
+          k_local_band_f64<<<npairs_c, nt, band_f64_smem(B), h.stream>>>(k, sptr, h.sub_dofs, B, h.bandK, h.bandM, lam, rho,
                                                            (double*)h.Lbuf, (double*)h.wpk, h.derr, rec_base);
         }
       }

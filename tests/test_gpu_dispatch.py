@@ -23,6 +23,33 @@ def _partition(lists):
     return B.PartitionArrays(ptr, np.concatenate(lists).astype(np.int32), None, 0)
 
 
+def _strips(window):
+    """A pencil whose grid rows are as long as the local window asks, with a full-rank interpolation."""
+    nx = window - 1
+    pb = B.problem_create("p1_2d", (nx, 12), (1.0, 12.0 / nx), (nx, 12), 1)
+    n = pb.K.n_rows
+    ix, iy = np.arange(n) % (nx - 1) + 1, np.arange(n) // (nx - 1) + 1
+    hat = lambda t, c: np.maximum(0.0, 1.0 - np.abs(t - c) * 4)  # noqa: E731
+    cols = [hat(ix / nx, a / 4) * hat(iy / 12, b / 4) for b in (1, 2, 3) for a in (1, 2, 3)]
+    pb.P = B.CsrArrays.from_scipy(sp.csr_matrix(np.array(cols).T))
+    return pb, nx - 1
+
+
+# ---- FP64 local solves --------------------------------------------------------------------------------------------
+
+# The widest FP64 window that is accepted, and the first one that is not.
+def test_fp64_widest_window():
+    for window, ok in ((168, True), (169, False)):
+        pb, _ = _strips(window)
+        part = _partition([np.arange(pb.K.n_rows)])
+        if ok:
+            assert B.Solver(pb.K, pb.M, pb.P, None, part, 2, precision=B.FP64).layout()["band_window"] == window
+        else:
+            with pytest.raises(B.BpjdError) as e:
+                B.Solver(pb.K, pb.M, pb.P, None, part, 2, precision=B.FP64)
+            assert e.value.code == B.ERR_UNSUPPORTED
+
+
 # ---- Gram products ------------------------------------------------------------------------------------------------
 
 # Several chunks to a block, the last one short, and tile counts that leave warps without one: 144 and 136 tiles

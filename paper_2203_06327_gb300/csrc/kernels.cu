@@ -832,8 +832,8 @@ __global__ void k_combine_rows(int64_t n, int k, int nin, Ptrs6 W, const double*
 }
 
 // ---------------------------------------------------------------------------
-// FP32 local solves of windows above the register tiers: one warp per
-// (subdomain l, column i) computes
+// Local solves of FP32 windows above the register tiers and of many narrow FP64
+// windows: one warp per (subdomain l, column i) computes
 //   w = (K_l - lambda_i M_l)^{-1} R_l rho_i
 // by a banded Cholesky factorisation streamed through a (B x B) window held
 // in shared memory (B = lower bandwidth + 1), with the forward substitution
@@ -844,10 +844,11 @@ __global__ void k_combine_rows(int64_t n, int k, int nin, Ptrs6 W, const double*
 // row j + B of the shifted band matrix into the freed slot.  Rows past n_l
 // are identity rows.  A pivot <= 0 sets err (Eq. (3.1) violated).
 // ---------------------------------------------------------------------------
+template <typename TP>
 __global__ void k_local_band(int npairs, int k, const int64_t* __restrict__ sub_ptr,
-                             const int32_t* __restrict__ sub_dofs, int B, const float* __restrict__ bandK,
-                             const float* __restrict__ bandM, const double* __restrict__ lam,
-                             const double* __restrict__ rho, float* __restrict__ Lbuf, float* __restrict__ wpk,
+                             const int32_t* __restrict__ sub_dofs, int B, const TP* __restrict__ bandK,
+                             const TP* __restrict__ bandM, const double* __restrict__ lam,
+                             const double* __restrict__ rho, TP* __restrict__ Lbuf, TP* __restrict__ wpk,
                              int32_t* err, int64_t rec_base) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x & 31;
@@ -855,47 +856,47 @@ __global__ void k_local_band(int npairs, int k, const int64_t* __restrict__ sub_
   const int pair = blockIdx.x * (blockDim.x >> 5) + wib;
   if (pair >= npairs) return;
   const int BB = B * B;
-  float* W = reinterpret_cast<float*>(smraw) + (size_t)wib * (BB + 3 * B);
-  float* rw = W + BB;   // right-hand side window
-  float* lc = rw + B;   // current column of L by slot
-  float* xs = lc + B;   // solution window (backward sweep)
+  TP* W = reinterpret_cast<TP*>(smraw) + (size_t)wib * (BB + 3 * B);
+  TP* rw = W + BB;   // right-hand side window
+  TP* lc = rw + B;   // current column of L by slot
+  TP* xs = lc + B;   // solution window (backward sweep)
   const int l = pair / k, i = pair % k;
   const int64_t off = sub_ptr[l];
   const int nl = (int)(sub_ptr[l + 1] - off);
   const int32_t* dofs = sub_dofs + off;
   const int b = B - 1;
-  const float lm = (float)lam[i];
-  float* Lp = Lbuf + ((size_t)(off - rec_base) * k + (size_t)i * nl) * B;
-  auto aval = [&](int p, int q) -> float {  // shifted local matrix entry, q <= p <= q + b
-    if (p >= nl) return (p == q) ? float(1) : float(0);
+  const TP lm = (TP)lam[i];
+  TP* Lp = Lbuf + ((size_t)(off - rec_base) * k + (size_t)i * nl) * B;
+  auto aval = [&](int p, int q) -> TP {  // shifted local matrix entry, q <= p <= q + b
+    if (p >= nl) return (p == q) ? TP(1) : TP(0);
     const size_t e = (size_t)(off + p) * B + (q - p + b);
     return bandK[e] - lm * bandM[e];
   };
   // initial window: rows 0..B-1
-  for (int e = lane; e < BB; e += 32) W[e] = float(0);
+  for (int e = lane; e < BB; e += 32) W[e] = TP(0);
   __syncwarp();
   for (int p = 0; p < B; ++p) {
     for (int e = lane; e <= b; e += 32) {
       int q = p - b + e;
       if (q < 0) continue;
-      float v = aval(p, q);
+      TP v = aval(p, q);
       W[(p % B) * B + (q % B)] = v;
       W[(q % B) * B + (p % B)] = v;
     }
     __syncwarp();
   }
-  for (int p = lane; p < B; p += 32) rw[p] = (p < nl) ? (float)rho[(int64_t)dofs[p] * k + i] : float(0);
+  for (int p = lane; p < B; p += 32) rw[p] = (p < nl) ? (TP)rho[(int64_t)dofs[p] * k + i] : TP(0);
   __syncwarp();
   for (int j = 0; j < nl; ++j) {
     const int s = j % B;
-    const float piv = W[s * B + s];
-    if (!(piv > float(0))) {
+    const TP piv = W[s * B + s];
+    if (!(piv > TP(0))) {
       if (lane == 0) atomicOr(err, 1);
       return;
     }
-    const float inv = float(1) / sqrt(piv);
-    for (int u = lane; u < B; u += 32) lc[u] = (u == s) ? float(0) : W[u * B + s] * inv;
-    const float yj = rw[s] * inv;
+    const TP inv = TP(1) / sqrt(piv);
+    for (int u = lane; u < B; u += 32) lc[u] = (u == s) ? TP(0) : W[u * B + s] * inv;
+    const TP yj = rw[s] * inv;
     __syncwarp();
     // L column j: slot 0 = 1/L_jj, slot t = L(j + t, j)
     for (int t = lane; t < B; t += 32) Lp[(size_t)j * B + t] = (t == 0) ? inv : lc[(j + t) % B];
@@ -922,25 +923,25 @@ __global__ void k_local_band(int npairs, int k, const int64_t* __restrict__ sub_
     const int pn = j + B;
     for (int e = lane; e <= b; e += 32) {
       int q = pn - b + e;  // q in j+1 .. j+B
-      float v = aval(pn, q);
+      TP v = aval(pn, q);
       W[s * B + (q % B)] = v;
       W[(q % B) * B + s] = v;
     }
-    if (lane == 0) rw[s] = (pn < nl) ? (float)rho[(int64_t)dofs[pn] * k + i] : float(0);
+    if (lane == 0) rw[s] = (pn < nl) ? (TP)rho[(int64_t)dofs[pn] * k + i] : TP(0);
     __syncwarp();
   }
   // backward substitution with L^T
-  for (int u = lane; u < B; u += 32) xs[u] = float(0);
+  for (int u = lane; u < B; u += 32) xs[u] = TP(0);
   __syncwarp();
   for (int j = nl - 1; j >= 0; --j) {
-    const float* row = Lp + (size_t)j * B;
-    float part = 0;
+    const TP* row = Lp + (size_t)j * B;
+    TP part = 0;
     for (int t = 1 + lane; t < B; t += 32) {
       if (j + t < nl) part += row[t] * xs[(j + t) % B];
     }
     part = warp_sum(part);
     if (lane == 0) {
-      float xj = (wpk[(off + j) * k + i] - part) * row[0];
+      TP xj = (wpk[(off + j) * k + i] - part) * row[0];
       xs[j % B] = xj;
       wpk[(off + j) * k + i] = xj;
     }
@@ -994,7 +995,7 @@ __global__ void __launch_bounds__(kBandF64Threads) k_local_band_f64(int k, const
   // slot of this thread (B: the right-hand side; threads past it only take part in the
   // window update); the slots sit in other warps from one block to the next, so that the
   // quarters of an SM share the per-slot work of its blocks
-  int u = tid + 32 * (blockIdx.x & 3);
+  int u = tid + 32 * ((blockIdx.x & 3) % (NT >> 5));
   u -= (u >= NT) ? NT : 0;
   const bool own = u < B;
   const int l = blockIdx.x / k, i = blockIdx.x % k;
@@ -1126,7 +1127,7 @@ __global__ void __launch_bounds__(kBandF64Threads) k_local_band_f64(int k, const
   // backward substitution by one warp (another SM quarter from one block to the next): lane t
   // sums the products of entries 1 + t, 33 + t, .. of record j with the solved rows, a
   // butterfly adds the lanes; record, y and 1/L_jj are loaded two rows ahead
-  if ((tid >> 5) != (int)(blockIdx.x & 3)) return;
+  if ((tid >> 5) != (int)(blockIdx.x & 3) % (NT >> 5)) return;
   constexpr int NC = kBandF64Record;
   const int lane = tid & 31;
   double* xs = lc;  // [B] solved rows by slot
@@ -3378,6 +3379,10 @@ bool can_reuse_factors(const Handle& h) {
   }
 }
 
+// FP64 local solves: widest windows of one warp per pair and of two-warp CTAs, and the pairs
+// from which on one warp per pair is taken (launch_local has the measurements)
+constexpr int kOneWarpWindow = 16, kTwoWarpWindow = 20, kOneWarpPairs = 14 * 152;
+
 // The local part of Eq. (3.3): mode kLocalFull factorises every (subdomain, shift)
 // pair and solves (chunk by chunk); kLocalReuse runs the forward and backward
 // sweeps on stored factors; the three single-kernel modes serve the captured
@@ -3512,21 +3517,33 @@ int launch_local(Handle& h, const double* rho, const double* lam, int mode) {
 #undef BPJD_LOCAL_TILE
 #undef BPJD_LOCAL_WIDE
       } else {
+        // one warp per pair: windows above the FP32 tiers, and FP64 windows up to kOneWarpWindow
+        // of more pairs than one wave of CTAs (14 of two warps on each SM), where the chain of a
+        // step is hidden by other pairs and a CTA per pair only adds barriers and idle lanes.
+        // us per application, one warp / CTA of two warps / of four (GB300): window 1, 261,121
+        // pairs 493 / 780 / 1021; window 10, 4096 pairs 579 / 640 / 737, 1024 pairs 281 / 206 / 217;
+        // window 12, 2028 pairs 527 / 485 / 566, 2704 pairs 653 / 931 / 813; window 16, 1369
+        // pairs 907 / 665 / 1081, 16,428 pairs 6568 / 6598 / 8267; window 20, 10,092 pairs 7729 /
+        // 7420 / 8452.  Two warps up to kTwoWarpWindow: a step has too few entries for four
+        // (window 26, 9 pairs: 1118, four 1010)
+        auto one_warp = [&](auto tag, auto* bK, auto* bM) {
+          using T = decltype(tag);
+          const size_t per_warp = (size_t)(B * B + 3 * B) * sizeof(T);
+          const int wpb = (int)std::max<size_t>(1, std::min<size_t>(4, (200 * 1024) / per_warp));
+          allow_dynamic_smem((const void*)k_local_band<T>);
+          k_local_band<T><<<(npairs_c + wpb - 1) / wpb, 32 * wpb, per_warp * wpb, h.stream>>>(
+              npairs_c, k, sptr, h.sub_dofs, B, bK, bM, lam, rho, (T*)h.Lbuf, (T*)h.wpk, h.derr, rec_base);
+        };
         if (f32) {
-          const size_t per_warp = (size_t)(B * B + 3 * B) * sizeof(float);
-          int wpb = (int)std::max<size_t>(1, std::min<size_t>(4, (200 * 1024) / per_warp));
-          size_t sm = per_warp * wpb;
-          int blocks = (npairs_c + wpb - 1) / wpb;
-          allow_dynamic_smem((const void*)k_local_band);
-          k_local_band<<<blocks, 32 * wpb, sm, h.stream>>>(npairs_c, k, sptr, h.sub_dofs, B, h.bandKf, h.bandMf, lam,
-                                                           rho, (float*)h.Lbuf, (float*)h.wpk, h.derr, rec_base);
+          one_warp(float(), h.bandKf, h.bandMf);
+        } else if (B <= kOneWarpWindow && npairs_c > kOneWarpPairs) {
+          one_warp(double(), h.bandK, h.bandM);
         } else {
-          // four warps (one per SM quarter), six when the window has more rows
-          const int nt = std::max(128, (B + 32) / 32 * 32);
+          const int nt = B <= kTwoWarpWindow ? 64 : std::max(128, (B + 32) / 32 * 32);
           if (B > kBandF64Max) return (int)cudaErrorInvalidValue;
           allow_dynamic_smem((const void*)k_local_band_f64);
-          k_local_band_f64<<<npairs_c, nt, band_f64_smem(B), h.stream>>>(k, sptr, h.sub_dofs, B, h.bandK, h.bandM, lam, rho,
-                                                           (double*)h.Lbuf, (double*)h.wpk, h.derr, rec_base);
+          k_local_band_f64<<<npairs_c, nt, band_f64_smem(B), h.stream>>>(
+              k, sptr, h.sub_dofs, B, h.bandK, h.bandM, lam, rho, (double*)h.Lbuf, (double*)h.wpk, h.derr, rec_base);
         }
       }
     }
@@ -3557,7 +3574,8 @@ int prime_kernel_attributes(Handle& h) {
     case 152: tier(std::integral_constant<int, 152>()); break;
     default: break;
   }
-  allow_dynamic_smem((const void*)k_local_band);
+  allow_dynamic_smem((const void*)k_local_band<float>);
+  allow_dynamic_smem((const void*)k_local_band<double>);
   allow_dynamic_smem((const void*)k_local_band_f64);
   return (int)cudaGetLastError();
 }

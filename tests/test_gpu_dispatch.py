@@ -23,6 +23,16 @@ def _partition(lists):
     return B.PartitionArrays(ptr, np.concatenate(lists).astype(np.int32), None, 0)
 
 
+def _boxes(nx, ny, m):
+    """Dofs of boxes of m x m grid points of an (nx - 1) x (ny - 1) grid, row by row."""
+    out = []
+    for b in range(0, ny - 1, m):
+        for a in range(0, nx - 1, m):
+            r, c = np.arange(b, min(ny - 1, b + m)), np.arange(a, min(nx - 1, a + m))
+            out.append((r[:, None] * (nx - 1) + c[None]).ravel())
+    return out
+
+
 def _strips(window):
     """A pencil whose grid rows are as long as the local window asks, with a full-rank interpolation."""
     nx = window - 1
@@ -35,7 +45,34 @@ def _strips(window):
     return pb, nx - 1
 
 
+def _apply(sv, rho, lam):
+    Z = torch.empty(rho.shape, dtype=torch.float64, device=DEV)
+    sv.apply_preconditioner(torch.tensor(rho, device=DEV), torch.tensor(lam, device=DEV), Z)
+    return Z.cpu().numpy()
+
+
 # ---- FP64 local solves --------------------------------------------------------------------------------------------
+
+# Narrow FP64 windows take one warp per pair from 2129 pairs on, a CTA per pair below: the same bits either way.
+# A small scratch cuts the second handle's subdomains into chunks below the line.  Windows of one row, of the last
+# two before the rule's end (16) and of the first ones past it, where both handles run the CTA kernel.
+@pytest.mark.parametrize("m,window", [(1, 1), (4, 6), (13, 15), (14, 16), (15, 17)])
+def test_fp64_narrow_windows_same_bits_either_way(m, window):
+    nx = 14 * m + 2 if m > 1 else 34  # the last boxes of a row are one dof wide
+    pb = B.problem_create("p1_2d", (nx, nx), (1.0, 1.0), (2, 2), 1)
+    lists = _boxes(nx, nx, m)
+    k = 2129 // len(lists) + 1
+    assert len(lists) * k > 2128 and k <= 32
+    n = pb.K.n_rows
+    rng = np.random.default_rng(m)
+    pb.P = B.CsrArrays.from_scipy(sp.csr_matrix(rng.uniform(0.0, 1.0, (n, k + 1))))
+    rho, lam = rng.standard_normal((n, k)), np.linspace(1.0, 12.0, k)
+    one = B.Solver(pb.K, pb.M, pb.P, None, _partition(lists), k, precision=B.FP64)
+    assert one.layout()["band_window"] == window
+    few = B.Solver(pb.K, pb.M, pb.P, None, _partition(lists), k, precision=B.FP64,
+                   local_scratch_bytes=8 * m * m * k * window * (len(lists) // 3))
+    np.testing.assert_array_equal(_apply(one, rho, lam), _apply(few, rho, lam))
+
 
 # The widest FP64 window that is accepted, and the first one that is not.
 def test_fp64_widest_window():

@@ -508,19 +508,19 @@ extern "C" int bpjd_setup(const bpjd_csr* A, const bpjd_csr* M, const bpjd_csr* 
       CK(dalloc(*h, &h->bandKf, nb));
       CK(dalloc(*h, &h->bandMf, nb));
       if (h->same_pattern) {
-        CKI(launch_band_fill(*h, h->A, h->M.val, nullptr, nullptr, h->bandKf, h->bandMf));
+        CKI(launch_band_fill(*h, h->A, h->M.val, nullptr, nullptr, h->bandKf, h->bandMf, true));
       } else {
-        CKI(launch_band_fill(*h, h->A, nullptr, nullptr, nullptr, h->bandKf, nullptr));
-        CKI(launch_band_fill(*h, h->M, nullptr, nullptr, nullptr, h->bandMf, nullptr));
+        CKI(launch_band_fill(*h, h->A, nullptr, nullptr, nullptr, h->bandKf, nullptr, true));
+        CKI(launch_band_fill(*h, h->M, nullptr, nullptr, nullptr, h->bandMf, nullptr, false));
       }
     } else {
       CK(dalloc(*h, &h->bandK, (size_t)sum_nl * h->B));
       CK(dalloc(*h, &h->bandM, (size_t)sum_nl * h->B));
       if (h->same_pattern) {
-        CKI(launch_band_fill(*h, h->A, h->M.val, h->bandK, h->bandM, nullptr, nullptr));
+        CKI(launch_band_fill(*h, h->A, h->M.val, h->bandK, h->bandM, nullptr, nullptr, false));
       } else {
-        CKI(launch_band_fill(*h, h->A, nullptr, h->bandK, nullptr, nullptr, nullptr));
-        CKI(launch_band_fill(*h, h->M, nullptr, h->bandM, nullptr, nullptr, nullptr));
+        CKI(launch_band_fill(*h, h->A, nullptr, h->bandK, nullptr, nullptr, nullptr, false));
+        CKI(launch_band_fill(*h, h->M, nullptr, h->bandM, nullptr, nullptr, nullptr, false));
       }
     }
     pt.mark("bands", h->stream);

@@ -253,9 +253,10 @@ inline size_t band_f64_smem(int B) {
 }
 // band rows of the local matrices of c (and of a second matrix with c's pattern,
 // values val2): FP32 rows of width max(B, Bpad), or panels, into outf / outf2 when outf
-// is set, else FP64 rows of width B into out / out2
+// is set, else FP64 rows of width B into out / out2.  ident: the panels' rows past a
+// subdomain's end are identity rows (of c: the stiffness, so that the shifted matrix has them)
 int launch_band_fill(Handle& h, const CsrDev& c, const double* val2, double* out, double* out2, float* outf,
-                     float* outf2);
+                     float* outf2, bool ident);
 int launch_galerkin(const CsrDev& A, const CsrDev& Msp, const CsrDev& P, const CsrDev& PT, double* KH,
                     double* MH, cudaStream_t s);
 

@@ -3729,7 +3729,7 @@ int launch_split_values(const double* v, int64_t nnz, float2* out, cudaStream_t 
 }
 
 int launch_band_fill(Handle& h, const CsrDev& c, const double* val2, double* out, double* out2, float* outf,
-                     float* outf2) {
+                     float* outf2, bool ident) {
   const unsigned blocks = (unsigned)((h.sum_nl + 127) / 128);
   if (outf && band_panels(h.Bpad)) {
     const size_t bytes = sizeof(float) * band_floats(h.sum_nl, h.nsub, h.B, h.Bpad);
@@ -3737,7 +3737,7 @@ int launch_band_fill(Handle& h, const CsrDev& c, const double* val2, double* out
     if (e == cudaSuccess && outf2) e = cudaMemsetAsync(outf2, 0, bytes, h.stream);
     if (e != cudaSuccess) return (int)e;
     k_band_panels<<<blocks, 128, 0, h.stream>>>(h.nsub, h.sum_nl, h.sub_ptr, h.sub_dofs, c.row_ptr, c.col, c.val, val2,
-                                                h.B, h.Bpad + 8, outf == h.bandKf ? 1 : 0, outf, outf2);
+                                                h.B, h.Bpad + 8, ident ? 1 : 0, outf, outf2);
   } else if (outf) {
     const int W = std::max(h.B, h.Bpad);
     k_band_fill<float><<<blocks, 128, 0, h.stream>>>(h.nsub, h.sum_nl, h.sub_ptr, h.sub_dofs, c.row_ptr, c.col, c.val,

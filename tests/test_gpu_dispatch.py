@@ -4,6 +4,7 @@ import ctypes as C
 
 import numpy as np
 import pytest
+import scipy.linalg as la
 import scipy.sparse as sp
 import scipy.sparse.linalg as spla
 
@@ -51,6 +52,14 @@ def _apply(sv, rho, lam):
     return Z.cpu().numpy()
 
 
+def _coarse(K, M, P, rho, lam):
+    """The coarse term of Eq. (3.3)."""
+    w, Phi = la.eigh((P.T @ K @ P).toarray(), (P.T @ M @ P).toarray())
+    y = (Phi.T @ (P.T @ rho)) / (w[:, None] - lam[None, :])
+    y[:len(lam)] = 0.0
+    return P @ (Phi @ y)
+
+
 # ---- FP64 local solves --------------------------------------------------------------------------------------------
 
 # Narrow FP64 windows take one warp per pair from 2129 pairs on, a CTA per pair below: the same bits either way.
@@ -85,6 +94,46 @@ def test_fp64_widest_window():
             with pytest.raises(B.BpjdError) as e:
                 B.Solver(pb.K, pb.M, pb.P, None, part, 2, precision=B.FP64)
             assert e.value.code == B.ERR_UNSUPPORTED
+
+
+# ---- FP32 local solves of the wide tiers (bands by column panels) -------------------------------------------------
+
+# Windows at both ends of the tiers 64, 96 and 152; subdomains of 1, 5, 8 and 9 dofs (below a panel, a panel, one row
+# more) between wide ones of every remainder modulo 8; M with K's pattern and a diagonal M (two passes over the bands).
+# Tolerance: a banded Cholesky solve in FP32 has a relative error of at most B kappa 2^-24 (kappa of the diagonally
+# scaled matrix) in the 2-norm; FP32 prolongation and restriction add 1e-6 of the largest entry.
+@pytest.mark.parametrize("lumped", [False, True], ids=["consistent", "lumped"])
+@pytest.mark.parametrize("window", [49, 64, 65, 96, 129, 152])
+def test_wide_windows_short_subdomains(window, lumped):
+    pb, row = _strips(window)
+    if lumped:
+        M = _scipy(pb.M)
+        pb.M = B.CsrArrays.from_scipy(sp.csr_matrix(sp.diags(np.asarray(M.sum(axis=1)).ravel())))
+    n = pb.K.n_rows
+    lists, at = [], 0
+    for extra, short in zip(range(8), (1, 5, 8, 9, 1, 5, 8, 9)):
+        size = 2 * row + extra
+        lists += [np.arange(at, at + size), np.arange(at + 3, at + 3 + short)]
+        at += row
+    lists += [np.arange(at, n), np.arange(n - 1, n)]
+    k = 2
+    rng = np.random.default_rng(window)
+    rho, lam = rng.standard_normal((n, k)), np.array([1.0, 9.0])
+    K, M, P = _scipy(pb.K), _scipy(pb.M), _scipy(pb.P)
+    ref, tol = _coarse(K, M, P, rho, lam), np.zeros((n, k))
+    for d in lists:
+        Kl, Ml = K[d][:, d].toarray(), M[d][:, d].toarray()
+        for i in range(k):
+            A = Kl - lam[i] * Ml
+            s = 1.0 / np.sqrt(np.diag(A))
+            ev = la.eigvalsh(s[:, None] * A * s)
+            w = la.solve(A, rho[d, i], assume_a="pos")
+            ref[d, i] += w
+            tol[d, i] += window * ev[-1] / ev[0] * 2.0 ** -24 * np.linalg.norm(w / s) * s.max()
+    tol += 1e-6 * np.abs(ref).max()
+    sv = B.Solver(pb.K, pb.M, pb.P, None, _partition(lists), k, precision=B.MIXED)
+    assert sv.layout()["band_window"] == window
+    assert np.all(np.abs(_apply(sv, rho, lam) - ref) <= tol)
 
 
 # ---- Gram products ------------------------------------------------------------------------------------------------

@@ -951,14 +951,15 @@ __global__ void k_local_band(int npairs, int k, const int64_t* __restrict__ sub_
 
 // ---------------------------------------------------------------------------
 // FP64 local solves: one CTA per (subdomain l, column i), the arithmetic of
-// k_local_band (column j eliminated with 1/L_jj = rsqrt(pivot), forward
+// k_local_band (column j eliminated with 1/L_jj = 1 / sqrt(pivot), forward
 // substitution fused in, records as written there).  The FP64 pipe of this GPU
 // takes a warp instruction every 64 cycles per SM quarter, whatever its active
 // lanes, so instructions on that pipe are the bound and everything else
 // (shared memory, barriers) is nearly free beside them:
 //   - the symmetric window is kept once (packed lower triangle by slot index,
-//     entry (u, v), u >= v, at u (u + 1) / 2 + v; the right-hand sides are its last row) and updated by all warps over
-//     the flat list of its entries, full lanes in every instruction;
+//     entry (u, v), u >= v, at u (u + 1) / 2 + v; the right-hand sides are its
+//     last row) and updated by all warps over the flat list of its entries, full
+//     lanes in every instruction;
 //   - the warp that updates the next pivot forms its reciprocal root while the
 //     other warps do the rest of the update;
 //   - band rows and right-hand sides enter from registers loaded a step and a
@@ -968,7 +969,7 @@ __global__ void k_local_band(int npairs, int k, const int64_t* __restrict__ sub_
 // right-looking backward sweep were 0.6 ms faster, and moved the iterates of a
 // slowly converging solve by 1e-9).
 // 64 subdomains of 32 x 32 cells, 12 columns, window 37 (GB300): one warp per pair
-// on a full square window 10.27 ms, this kernel 3.7 ms (the FP64 pipe and the chain
+// on a full square window 10.27 ms, this kernel 3.86 ms (the FP64 pipe and the chain
 // of a step; six pairs on some SMs against five on others)
 // ---------------------------------------------------------------------------
 constexpr int kPivotChunks = 16;
@@ -3646,8 +3647,8 @@ int launch_local_grouped(Handle* const* hs, const double* const* rho, const doub
                                         s>>>(gb, nbuf);
     } else {
       const size_t bsm = sizeof(float) * BwdShape<B>::smem_floats;
-      // wide tiers: each request's factorisation in a launch of its own (its register
-      // allocation is tuned for one subdomain-shift pair per CTA), on the shared stream
+      // wide tiers: each request's factorisation in a launch of its own, on the shared stream
+      // (a CTA takes one pair of one handle's panels; the kernel reads no segment table)
       for (int j = 0; j < gf.n; ++j) {
         const LocalSeg& q = gf.s[j];
         allow_dynamic_smem((const void*)k_local_factor_wide<B>);
